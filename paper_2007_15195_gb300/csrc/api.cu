@@ -304,7 +304,9 @@ uint32_t* lattice_for(vecchia_ctx* c, int64_t N) {
 
 // Built-in tile (measured on the 50x50 grid): mixed blocks of up to 32
 // variables run two points per lane (one vote per step for both), 4 warps up
-// to 21 variables and 8 above; FP64 one point, 4 warps.  Shift groups (a power
+// to 21 variables and 8 above; FP64 one point, up to 8 warps with the shifts
+// spread evenly (its function tables take 45 KB a CTA, so 16 resident warps want
+// two CTAs of 8: 55.6 against 58.2 ms with 4 warps at m = 20).  Shift groups (a power
 // of two, so S = 2^k splits evenly) until a launch has ~2048 CTA items, never
 // fewer shifts per item than warps (a warp without a unit idles); ~4096 items
 // for blocks of up to 16 variables, which fit more CTAs per SM.  Blocks
@@ -321,7 +323,8 @@ GenzTile default_tile(bool mixed, int64_t total_sites, int max_S, int bucket) {
         t.groups = 1;
         return t;
     }
-    t.warps = (mixed && dmax > 21) ? 8 : 4;
+    const int rounds = (max_S + 7) / 8;
+    t.warps = mixed ? (dmax > 21 ? 8 : 4) : (max_S + rounds - 1) / rounds;
     t.points = mixed ? 2 : 1;
     t.slices = 1;
     // small blocks fit more CTAs per SM: they want more items

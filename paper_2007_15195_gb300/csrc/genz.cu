@@ -35,6 +35,7 @@
 #include "cov.cuh"
 #include "special_f32.h"
 #include "special_f64.h"
+#include "special_fix.h"
 #include "vk_internal.h"
 
 namespace vk {
@@ -51,12 +52,22 @@ __device__ __forceinline__ void tri_index(int e, int& r, int& c) {
     c = e - r * (r + 1) / 2;
 }
 
+// FP64 path, step t: the lattice coordinate's multiplier round(g_t 2^64 / N),
+// the coefficient -L_{t+1,t} and 1/L_{t+1,t+1} as integers (below), the shift
+// that takes their product to z 2^58, and its value at |z| = 9.25.
+struct __align__(16) FixStep {
+    uint64_t G;
+    fix::Digits nlz, rdiag;
+    int64_t lim;
+    int shift, pad[3];
+};
+
 // Shared memory of a CTA: this fixed part, then (mixed path) the dynamic
 // tail dfix[S][DMAX] (the shifts in 32-bit fixed point) and
 // stepw[warps][DMAX] (per warp, the step constants of its current shift).
 template <int DMAX, bool MIXED>
 struct GenzSmem {
-    using T = typename std::conditional<MIXED, float, double>::type;
+    using T = typename std::conditional<MIXED, float, fix::Digits>::type;
     double A[DMAX][DMAX + 1];  // covariance block, overwritten by its Cholesky factor
     double bx[DMAX], by[DMAX], bu[DMAX];
     double diag[DMAX];
@@ -66,38 +77,34 @@ struct GenzSmem {
     //   Lup[t][r]  = L_{t+2+r,t}        coefficients of y_t in the later variables
     // MIXED multiplies each row v by kZs/L_vv (so the conditional mean arrives
     // standardised and times kZs = sqrt(log2(e)/2), the form its Phi takes);
-    // FP64 keeps them unscaled and multiplies the conditional mean by 1/L_vv
-    // (diag), one rounding more than the definition's division.
+    // FP64 keeps -L as integers of the row's scale (Lup; Lz in step), exact to
+    // 2^-60 of the row's largest possible sum, and multiplies the conditional mean
+    // by 1/L_vv, one rounding more than the definition's division.
     static constexpr int LS = (DMAX + 3) & ~3;  // row stride: 16-byte aligned rows
     __align__(16) T Lup[DMAX][LS];
-    __align__(16) T Lz[DMAX];
-    __align__(16) T up[DMAX];  // MIXED: kZs u_v / L_vv;  FP64: u_v
-    uint32_t gl[DMAX];         // FP64: g_t;  MIXED: round(g_t 2^32 / N)
-    uint64_t g64[MIXED ? 1 : DMAX];  // FP64: round(g_t 2^64 / N)
+    __align__(16) T Lz[MIXED ? DMAX : 1];
+    __align__(16) typename std::conditional<MIXED, float, int64_t>::type up[DMAX];  // MIXED: kZs u_v / L_vv
+    uint32_t gl[MIXED ? DMAX : 1];  // round(g_t 2^32 / N)
     double part_num[kMaxUnits], part_den[kMaxUnits];
     double e0, ec0;
     float le2_0;  // log2 e0 when e0 < 2^-64 (mixed path)
     int q, c, bad, flag;
+    // FP64: e0, each step's constants and each row's scale kL
+    fix::FixProb p0;
+    __align__(16) FixStep step[MIXED ? 1 : DMAX];
+    int scale[MIXED ? 1 : DMAX];
 };
 
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
-// FP64 path, per warp and step of its current shift: the lattice coordinate's
-// multiplier and shift in 64-bit fixed point (round(g_t 2^64 / N), Delta_t 2^64)
-// and the step's coefficient -L_{t+1,t} and 1/L_{t+1,t+1}.
-struct Step64 {
-    uint64_t G, D;
-    double nlz, rdiag;
-};
-
 // Bytes of shared memory for a CTA of `warps` warps on problems with <= max_S
 // shifts: the fixed part, then (mixed) the shifts in fixed point and the
-// per-warp step constants, or (FP64) the tail tables and the per-warp steps.
+// per-warp step constants, or (FP64) the function tables and each warp's shift.
 template <int DMAX, bool MIXED>
 constexpr size_t smem_bytes(int max_S, int warps) {
     return align16(sizeof(GenzSmem<DMAX, MIXED>)) +
            (MIXED ? align16((size_t)max_S * DMAX * 4) + (size_t)warps * DMAX * 16
-                  : align16(sizeof(special64::Tables64)) + (size_t)warps * DMAX * sizeof(Step64));
+                  : align16(sizeof(fix::FixTables)) + (size_t)warps * DMAX * sizeof(uint64_t));
 }
 
 extern __shared__ __align__(16) unsigned char vk_smem[];
@@ -114,13 +121,13 @@ __device__ __forceinline__ float4* stepw_of(int max_S, int warp) {
            warp * DMAX;
 }
 template <int DMAX>
-__device__ __forceinline__ special64::Tables64& tables64() {
-    return *reinterpret_cast<special64::Tables64*>(vk_smem + align16(sizeof(GenzSmem<DMAX, false>)));
+__device__ __forceinline__ fix::FixTables& fix_tables() {
+    return *reinterpret_cast<fix::FixTables*>(vk_smem + align16(sizeof(GenzSmem<DMAX, false>)));
 }
 template <int DMAX>
-__device__ __forceinline__ Step64* step64_of(int warp) {
-    return reinterpret_cast<Step64*>(vk_smem + align16(sizeof(GenzSmem<DMAX, false>)) +
-                                     align16(sizeof(special64::Tables64))) +
+__device__ __forceinline__ uint64_t* shift64_of(int warp) {
+    return reinterpret_cast<uint64_t*>(vk_smem + align16(sizeof(GenzSmem<DMAX, false>)) +
+                                       align16(sizeof(fix::FixTables))) +
            warp * DMAX;
 }
 
@@ -416,52 +423,79 @@ __device__ __forceinline__ void genz_points_fast(const GenzSmem<DMAX, true>& sm,
 }
 
 // ------------------------------- FP64 path ---------------------------------
+// The step in 64-bit fixed point (special_fix.h); FP64 only in the tails that
+// its tables leave out and in the two sums over points.
 
-// Lattice coordinate in 64-bit fixed point to a double: V 2^-63 for
-// 0 <= V <= 2^63, rounded to 53 bits (integer instructions only).
-__device__ __forceinline__ double fix63_to_f64(uint64_t V) {
-    if (V == 0) return 0.0;
-    const int lz = __clzll((long long)V);
-    const uint64_t m = V << lz;  // bit 63 set
-    const uint64_t bits = ((uint64_t)(1023 - lz) << 52) + ((m >> 11) & 0xFFFFFFFFFFFFFull) + ((m >> 10) & 1);
-    return __longlong_as_double((long long)bits);
+// |Phi^{-1}(s)| 2^57 of s = m 2^-64 2^-lz below 2^-32 (one step in 2^31 unless
+// the thresholds themselves are that deep): the FP64 quantile.
+__device__ __forceinline__ int64_t quantile_tail(uint64_t m, int lz) {
+    const double s = __longlong_as_double((long long)fix::to_bits(fix::FixFloat{m, lz}));
+    const double y = special64::phiinv_pq(special64::global_tables(), s, 1.0);
+    return __double2ll_rn(-y * 0x1p57);
 }
 
-// One FP64 step t (lattice coordinate t, variable t + 1 next) of a point:
-// update width W.  x = frac(k g_t / N + Delta_t) in 64-bit fixed point
-// X = k G_t + D_t mod 2^64; the tent w = 1 - |2x - 1| = |int64(X)| 2^-63
-// and |2x - 1| = 1 - w from the same integer.
-template <int DMAX, int W>
-__device__ __forceinline__ void fp64_step(const GenzSmem<DMAX, false>& sm, const special64::Tables64& tb,
-                                          const Step64& st, int t, uint32_t k, double (&R)[DMAX - 1], double& e,
-                                          double& ec) {
-    const uint64_t X = (uint64_t)k * st.G + st.D;
-    const uint64_t V = ((int64_t)X < 0) ? (0ull - X) : X;  // |int64(X)| <= 2^63
-    const double w = fix63_to_f64(V);
-    const double a = fix63_to_f64((1ull << 63) - V);
-    const double pp = w * e;
-    const double qq = fma(w, ec, a);
-    const double y = special64::phiinv_pq(tb, pp, qq);
-    const double* lup = sm.Lup[t];
-    const double acc = fma(st.nlz, y, R[0]);
-#pragma unroll
-    for (int r = 0; r < W; ++r) R[r] = fma(-lup[r], y, R[r + 1]);
-    special64::phi_pair(tb, acc * st.rdiag, e, ec);
+// Phi at z = hi 2^(shift - 58) <= -7: the FP64 tail.
+__device__ __forceinline__ void deep_prob(int64_t hi, int shift, fix::FixProb& p) {
+    double unused;
+    const double z = ldexp((double)hi, shift - 58);
+    const double t = special64::tail<false>(special64::global_tables(), -z, unused);
+    p = fix::prob_of((uint64_t)__double_as_longlong(t), true);
 }
 
-// Steps t <= t' < q in phases of update width W, W - step, ... (as the mixed path).
-template <int DMAX, int W>
-__device__ __forceinline__ void fp64_phases(const GenzSmem<DMAX, false>& sm, const special64::Tables64& tb,
-                                            const Step64* st, int t, int q, int c, uint32_t k,
-                                            double (&R)[DMAX - 1], double& e, double& ec, double& f, double& fc) {
-    constexpr int WN = W - phase_step(DMAX);
-    const int t_end = (WN > 0) ? max(t, min(q, q - 1 - WN)) : q;
-    for (int tt = t; tt < t_end; ++tt) {
-        f *= e;                   // e_0 ... e_tt
-        if (tt + 1 == c) fc = f;  // the c-dim CDF sample of the leading block
-        fp64_step<DMAX, W>(sm, tb, st[tt], tt, k, R, e, ec);
+// One step t (lattice coordinate t, variable t + 1 next) of a point whose
+// later variables are `later` = q - 1 - t (warp-uniform).  x = frac(k g_t / N +
+// Delta_t) in 64-bit fixed point X = k G_t + D_t.
+//
+// Bound by instruction issue: 385 instructions a step at m = 20 (60 IMAD.WIDE
+// at 4 cycles each, two or three additions a product), against 77 FP64 ones at
+// 76 cycles in the FP64 form.  50 x 50 grid, m = 20, N S = 65,536: 453 ms in
+// FP64, 55.5 ms so; m = 30 (N S = 16,384) 182 -> 24.9 ms; m = 50 (8,192)
+// 169 -> 37.6 ms.  One copy of the body serves every step and the updates run
+// in groups of four variables behind uniform branches: phases with a copy
+// each, as the mixed path has them, overran the instruction cache (94.6 ms
+// against 73 ms at that point), two or three phases padded more than they saved.
+template <int DMAX>
+__device__ __forceinline__ void fix_step(const GenzSmem<DMAX, false>& sm, const fix::FixTables& tb, uint64_t Dt,
+                                         int t, int later, uint32_t k, uint64_t K, int64_t (&R)[DMAX - 1],
+                                         fix::FixProb& e) {
+    const FixStep& st = sm.step[t];
+    const uint64_t w = fix::tent((uint64_t)k * st.G + Dt);
+    const uint64_t pp = fix::umul_hi(w, e.E);
+    const int64_t upper = (int64_t)pp >> 63;  // all ones where 1 - w e is the smaller
+    const uint64_t s = pp ^ (uint64_t)upper;
+    int lz = fix::clz32((uint32_t)(s >> 32));
+    uint64_t m = s << lz;
+    fix::Digits X;
+    const int row = fix::quant_row(m, min(lz, fix::kQShared), X);
+    int64_t y = fix::poly(tb.quant[row], X, fix::kQShift3, K);
+    if (lz > fix::kQShared) {
+        fix::small_s(w, e, upper == 0, m, lz);
+        if (lz <= 31) {
+            const int far = fix::quant_row(m, lz, X);
+            y = fix::poly(fix::kQuantRow[far], X, fix::kQShift3, K);
+        } else
+            y = quantile_tail(m, lz);
     }
-    if constexpr (WN > 0) fp64_phases<DMAX, WN>(sm, tb, st, t_end, q, c, k, R, e, ec, f, fc);
+    const fix::Digits Y = fix::digits((y ^ ~upper) - ~upper);
+    const int64_t acc = fix::mul_add(st.nlz, Y, R[0], K);
+    const fix::Digits* lup = sm.Lup[t];
+#pragma unroll
+    for (int r0 = 0; r0 < DMAX - 2; r0 += 4) {
+        if (later <= r0) break;
+#pragma unroll
+        for (int r = r0; r < r0 + 4 && r < DMAX - 2; ++r) R[r] = fix::mul_add(lup[r], Y, R[r + 1], K);
+    }
+    const int64_t hi = fix::mul_add(st.rdiag, fix::digits(acc), -fix::kMulBias, K);
+    const int64_t neg = hi >> 63;
+    const int64_t a = (hi ^ neg) - neg;
+    const uint64_t A = (uint64_t)a << (st.shift & 63);  // |z| 2^58
+    const bool big = a >= st.lim;
+    uint64_t T;
+    fix::tail_poly(tb.tail, tb.meta, A, e.mt, e.et, K);
+    T = e.mt >> e.et;
+    if (big) e.mt = T = 0;  // z >= 9.25: Phi = 1 to 2^-66
+    e.E = T ^ (uint64_t)~neg;
+    if (hi < 0 && (big || A >= (7ull << 58))) deep_prob(hi, st.shift, e);
 }
 
 // 2^64 g / N rounded to the nearest integer (g < N < 2^32), by two steps of
@@ -472,30 +506,65 @@ __device__ __forceinline__ uint64_t fix64_ratio(uint32_t g, uint64_t N) {
     return (q1 << 32) + q2 + ((2 * r2 >= N) ? 1u : 0u);
 }
 
+// The scale of row v (v >= 1) and its step constants, one thread a row.  With
+// B above |u_v| + 38.6 sum_t |L_vt| (|y| < 38.6: the quantile is clamped at
+// 2^-1000) and 2^e <= B < 2^(e + 1), L_vt is kept as an integer of 2^-kL,
+// kL = 67 - e (|L_vt| < B / 38.6: below 2^63), and sums as integers of
+// 2^(7 - kL) (below 2^61).  u_v is clamped where Phi is 0 or 1 whatever the
+// y_t (NaN as +inf, as the FP64 functions took it).
 template <int DMAX>
-__device__ __forceinline__ void genz_points_fp64(const GenzSmem<DMAX, false>& sm, const ProbDev& P,
+__device__ __forceinline__ void fix_row(GenzSmem<DMAX, false>& sm, int v, uint32_t g, uint64_t N) {
+    const double lvv = sm.A[v][v], rd = 1.0 / lvv;
+    double sum = 0.0;
+    for (int t = 0; t < v; ++t) sum += fabs(sm.A[v][t]);
+    const double reach = 38.6 * sum, umax = reach + 39.0 * lvv;
+    const double u = fmax(-umax, fmin(umax, sm.bu[v]));
+    const double B = fmax(fabs(u) + reach, 32.0 * lvv);
+    const int e = ilogb(B), kL = 67 - e;
+    const long long rb = __double_as_longlong(rd);
+    const int S = (int)((rb >> 52) & 0x7ff) - 1023 + e;
+    sm.scale[v] = kL;
+    sm.up[v] = __double2ll_rn(ldexp(u, kL - 7)) - v * fix::kMulBias;  // v products are added
+    FixStep& st = sm.step[v - 1];
+    st.G = fix64_ratio(g, N);
+    st.nlz = fix::digits(__double2ll_rn(ldexp(-sm.A[v][v - 1], kL)));
+    st.rdiag = fix::digits(((rb & 0xfffffffffffffll) | (1ll << 52)) << 10);  // 1/L_vv = this 2^(S - e - 62)
+    st.lim = S <= 56 ? 37ll << (56 - S) : S < 62 ? (37 + (1 << (S - 56)) - 1) >> (S - 56) : 1;
+    st.shift = S;
+}
+
+template <int DMAX>
+__device__ __forceinline__ void genz_points_fp64(const ProbDev& P,
                                                  int q, int c, int s, int64_t k_begin, int64_t k_end,
                                                  double& acc_num, double& acc_den) {
-    constexpr int W0 = (DMAX - 2 > 0) ? DMAX - 2 : 1;
     const int lane = threadIdx.x & 31;
-    const special64::Tables64& tb = tables64<DMAX>();
-    Step64* st = step64_of<DMAX>(threadIdx.x >> 5);
+    // The shared memory's base as a value the compiler keeps in a register
+    // (it forms the address of the array itself anew at every use).
+    uint32_t base;
+    asm volatile("mov.u32 %0, %1;" : "=r"(base) : "r"((uint32_t)__cvta_generic_to_shared(vk_smem)));
+    const unsigned char* smem = (const unsigned char*)__builtin_assume_aligned(__cvta_shared_to_generic(base), 16);
+    const GenzSmem<DMAX, false>& sm = *reinterpret_cast<const GenzSmem<DMAX, false>*>(smem);
+    const fix::FixTables& tb = *reinterpret_cast<const fix::FixTables*>(smem + align16(sizeof(GenzSmem<DMAX, false>)));
+    uint64_t* D = shift64_of<DMAX>(threadIdx.x >> 5);
+    const uint64_t K = fix::opaque_mid();
     const double* dl = P.delta + (int64_t)s * P.dim;
     __syncwarp();
-    for (int t = lane; t < q; t += 32) {
-        // Delta = M 2^-53 exactly (53-bit shifts): D = M 2^11
-        const uint64_t M = (uint64_t)__double2ull_rn(dl[t] * 9007199254740992.0);
-        st[t] = Step64{sm.g64[t], M << 11, -sm.Lz[t], sm.diag[t + 1]};
-    }
+    for (int t = lane; t < q; t += 32)  // Delta = M 2^-53 exactly (53-bit shifts): D = M 2^11
+        D[t] = (uint64_t)__double2ull_rn(dl[t] * 9007199254740992.0) << 11;
     __syncwarp();
     for (int64_t k = k_begin + lane; k < k_end; k += 32) {
-        double R[DMAX - 1];
+        int64_t R[DMAX - 1];
 #pragma unroll
         for (int r = 0; r < DMAX - 1; ++r) R[r] = sm.up[1 + r];
-        double e = sm.e0, ec = sm.ec0, f = 1.0, fc = 1.0;
-        fp64_phases<DMAX, W0>(sm, tb, st, 0, q, c, (uint32_t)k, R, e, ec, f, fc);
-        acc_den += fc;
-        acc_num += f * e;
+        fix::FixProb e = sm.p0;
+        fix::FixFloat f = fix::prob(e), fc = f;  // c = 1: e_0
+        for (int t = 0; t < q; ++t) {
+            if (t + 1 == c) fc = f;  // e_0 ... e_{c-1}: the c-dim CDF sample of the leading block
+            fix_step<DMAX>(sm, tb, D[t], t, q - 1 - t, (uint32_t)k, K, R, e);
+            f = fix::times(f, e);  // e_0 ... e_{t+1}
+        }
+        acc_den += __longlong_as_double((long long)fix::to_bits(fc));
+        acc_num += __longlong_as_double((long long)fix::to_bits(f));
     }
 }
 
@@ -565,7 +634,9 @@ __device__ __forceinline__ void item_of(const ItemSrc& src, int it, int2& ps, in
 // MODE: 0 = FP64, 1 = mixed fast form, 2 = mixed log-space form.
 constexpr int kModeFP64 = 0, kModeFast = 1, kModeSafe = 2;
 
-// Register cap per thread: the fast mixed loop keeps DMAX - 1 partial sums per
+// Register cap per thread: the FP64 step at up to 13 variables runs best with
+// 20 warps an SM (m = 10: 8.0 against 8.4 ms at 128 registers); from 14 on more
+// warps than 16 lose to spills.  The fast mixed loop keeps DMAX - 1 partial sums per
 // point in registers; capping the rest raises the number of resident warps.
 // Blocks above 32 variables run one point per lane with up to 128 registers
 // (fast) or 255 (FP64 and log-space forms, whose partial sums are wider), and
@@ -584,7 +655,7 @@ constexpr int kModeFP64 = 0, kModeFast = 1, kModeSafe = 2;
 #endif
 __host__ __device__ constexpr int reg_cap(int dmax, int p, int mode) {
     return dmax > 32            ? (mode == kModeFast ? 128 : 255)
-           : mode != kModeFast ? 128
+           : mode != kModeFast ? (mode == kModeFP64 && dmax <= 13 ? 96 : 128)
            : p == 1            ? (dmax <= 16 ? VK_CAP_P1_SMALL : VK_CAP_P1_LARGE)
                                : (dmax <= 16 ? VK_CAP_P2_SMALL : VK_CAP_P2_LARGE);
 }
@@ -649,7 +720,12 @@ __global__ void __launch_bounds__(max_threads(DMAX, P, MODE)) __maxnreg__(reg_ca
     const int n_warps = blockDim.x >> 5;
 
     if constexpr (!MIXED) {
-        special64::load_tables(tables64<DMAX>());
+        fix::FixTables& tb = fix_tables<DMAX>();
+        for (int i = threadIdx.x; i < fix::kQShared * fix::kQSub; i += blockDim.x) tb.quant[i] = fix::kQuantRow[i];
+        for (int i = threadIdx.x; i < fix::kTRows; i += blockDim.x) {
+            tb.tail[i] = fix::kTailRow[i];
+            tb.meta[i] = fix::kTailMeta[i];
+        }
         __syncthreads();
     }
     const int n_run = src.dev_count ? min(*src.dev_count, src.n_items) : src.n_items;
@@ -744,46 +820,47 @@ __global__ void __launch_bounds__(max_threads(DMAX, P, MODE)) __maxnreg__(reg_ca
 
         if (!sm.bad) {
             // ---- derived tables for the recursion ----
-            // (one FP64 reciprocal 1/L_vv per row; mixed: each row scaled by
+            // (mixed: one FP64 reciprocal 1/L_vv per row, each row scaled by
             // kZs/L_vv, so the recursion's conditional means arrive as the
-            // kZs z that its Phi takes)
+            // kZs z that its Phi takes; FP64: integers of each row's scale)
             constexpr int LS = GenzSmem<DMAX, MIXED>::LS;
             const int d = q + 1;
-            for (int v = threadIdx.x; v < DMAX; v += blockDim.x)
-                sm.diag[v] = (v < d) ? (MIXED ? special::kZsD : 1.0) / sm.A[v][v] : 0.0;
+            if constexpr (MIXED) {
+                for (int v = threadIdx.x; v < DMAX; v += blockDim.x)
+                    sm.diag[v] = (v < d) ? special::kZsD / sm.A[v][v] : 0.0;
+            } else {
+                for (int v = threadIdx.x; v < DMAX; v += blockDim.x) {
+                    if (v >= 1 && v < d)
+                        fix_row<DMAX>(sm, v, Pd.g[v - 1], (uint64_t)Pd.N);
+                    else
+                        sm.up[v] = 0;
+                }
+                if (threadIdx.x == 0) {
+                    const double z0 = sm.bu[0] / sm.A[0][0];
+                    sm.p0 = fix::prob_of((uint64_t)__double_as_longlong(z0 < 0.0 ? sm.e0 : sm.ec0), z0 < 0.0);
+                }
+            }
             __syncthreads();
             for (int x = threadIdx.x; x < DMAX * LS; x += blockDim.x) {
                 const int t = x / LS, r = x % LS, v = t + 2 + r;
-                T val = (T)0;
+                T val = T();
                 if (t < q && v < d) {
                     if constexpr (MIXED)
                         val = (T)(sm.A[v][t] * sm.diag[v]);
                     else
-                        val = sm.A[v][t];
+                        val = fix::digits(__double2ll_rn(ldexp(-sm.A[v][t], sm.scale[v])));
                 }
                 sm.Lup[t][r] = val;
             }
-            for (int v = threadIdx.x; v < DMAX; v += blockDim.x) {
-                T val = (T)0, lz = (T)0;
-                if (v < d) {
-                    if constexpr (MIXED)
-                        val = (T)(sm.bu[v] * sm.diag[v]);
-                    else
-                        val = sm.bu[v];
-                }
-                if (v < q) {
-                    if constexpr (MIXED)
-                        lz = (T)(sm.A[v + 1][v] * sm.diag[v + 1]);
-                    else
-                        lz = sm.A[v + 1][v];
-                }
-                sm.up[v] = val;
-                sm.Lz[v] = lz;
-                if (v < q) sm.gl[v] = MIXED ? Pd.gfix[v] : Pd.g[v];
-                if constexpr (!MIXED)
-                    if (v < q) sm.g64[v] = fix64_ratio(Pd.g[v], (uint64_t)Pd.N);
-            }
             if constexpr (MIXED) {
+                for (int v = threadIdx.x; v < DMAX; v += blockDim.x) {
+                    T val = (T)0, lz = (T)0;
+                    if (v < d) val = (T)(sm.bu[v] * sm.diag[v]);
+                    if (v < q) lz = (T)(sm.A[v + 1][v] * sm.diag[v + 1]);
+                    sm.up[v] = val;
+                    sm.Lz[v] = lz;
+                    if (v < q) sm.gl[v] = Pd.gfix[v];
+                }
                 for (int x = threadIdx.x; x < S * DMAX; x += blockDim.x) {
                     const int s = x / DMAX, t = x % DMAX;
                     dfix_row<DMAX>(s)[t] = (t < q) ? Pd.dfix[(int64_t)s * Pd.dim + t] : 0u;
@@ -808,7 +885,7 @@ __global__ void __launch_bounds__(max_threads(DMAX, P, MODE)) __maxnreg__(reg_ca
                 else if constexpr (MODE == kModeSafe)
                     genz_points_safe<DMAX, P>(sm, q, c, s, k0, k1, an, ad);
                 else
-                    genz_points_fp64<DMAX>(sm, Pd, q, c, s, k0, k1, an, ad);
+                    genz_points_fp64<DMAX>(Pd, q, c, s, k0, k1, an, ad);
                 an = warp_sum(an);
                 ad = warp_sum(ad);
                 if (lane == 0) {
@@ -839,6 +916,9 @@ __global__ void __launch_bounds__(max_threads(DMAX, P, MODE)) __maxnreg__(reg_ca
                 if constexpr (MIXED) {
                     vn *= sm.e0;
                     vd *= sm.e0;
+                }
+                if constexpr (!MIXED) {
+                    if (sm.e0 != sm.e0) vn = vd = sm.e0;  // a NaN threshold
                 }
                 if (c == 0) vd = 1.0;  // no conditioning set: the term is the joint CDF itself
                 if constexpr (MIXED) {

@@ -38,6 +38,13 @@ struct Tables64 {
     double E[1 << kExpBits];
 };
 
+// The same tables where they are read rarely: global memory.
+struct GlobalTables64 {
+    const double (*R)[kRStride];
+    const double* E;
+};
+__device__ __forceinline__ GlobalTables64 global_tables() { return GlobalTables64{kR, kExp2Frac}; }
+
 // Copy the tables into shared memory (all threads of the CTA; caller syncs).
 __device__ __forceinline__ void load_tables(Tables64& t) {
     const double* r = &kR[0][0];
@@ -66,8 +73,8 @@ __device__ __forceinline__ double abs_bits(double x) { return __longlong_as_doub
 __device__ __forceinline__ bool sign_bit(double x) { return bits(x) < 0; }
 
 // T = Phi(-a) for a >= 0, and (WANT_PHI) phi(a) = exp(-a^2/2)/sqrt(2 pi).
-template <bool WANT_PHI>
-__device__ __forceinline__ double tail(const Tables64& tb, double a, double& phi) {
+template <bool WANT_PHI, class TB>
+__device__ __forceinline__ double tail(const TB& tb, double a, double& phi) {
     if (bits(a) >= 0x4043600000000000ll) {  // a >= 38.75 (and inf, NaN): Phi(-a) below the smallest double
         if constexpr (WANT_PHI) phi = 0.0;
         return 0.0;
@@ -114,7 +121,8 @@ __device__ __forceinline__ double tail(const Tables64& tb, double a, double& phi
 }
 
 // Phi(z) and 1 - Phi(z), the smaller one from the tail to full precision.
-__device__ __forceinline__ void phi_pair(const Tables64& tb, double z, double& e, double& ec) {
+template <class TB>
+__device__ __forceinline__ void phi_pair(const TB& tb, double z, double& e, double& ec) {
     double unused;
     const double t = tail<false>(tb, abs_bits(z), unused);
     const double u = 1.0 - t;
@@ -150,7 +158,8 @@ __device__ __forceinline__ double to_f64_pos(float f) {
 
 // Phi^{-1}(p) given p and q = 1 - p: from the smaller of the two, clamped at
 // 2^-1000 (as the definition's quantile).
-__device__ __forceinline__ double phiinv_pq(const Tables64& tb, double p, double q) {
+template <class TB>
+__device__ __forceinline__ double phiinv_pq(const TB& tb, double p, double q) {
     const double lo = 9.3326361850321887899e-302;  // 2^-1000
     const double pc = max_nonneg(p, lo), qc = max_nonneg(q, lo);  // p, q >= 0
     const bool lower = bits(pc) <= bits(qc);
