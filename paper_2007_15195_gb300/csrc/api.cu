@@ -988,8 +988,8 @@ int vecchia_order(vecchia_ctx* c, const double* sites, int64_t D, int kind, int3
     // with no context both arrays are host memory and the ordering runs on the host
     const bool dev_in = c && is_device_ptr(sites), dev_out = c && is_device_ptr(perm);
     if (c && (dev_in || dev_out) && cudaSetDevice(c->device) != cudaSuccess) return VECCHIA_ERR_CUDA;
-    if (c && kind == VECCHIA_ORDER_XY && dev_in && dev_out && D <= vk::kOrderXyDeviceMax) {
-        // XY on the device: each site's rank counts the smaller (x, y, index) keys
+    if (c && kind == VECCHIA_ORDER_XY && dev_in && dev_out) {
+        // XY on the device
         int st = ensure_arena(c, vk::order_xy_scratch_bytes(D));
         if (st != VECCHIA_OK) return st;
         const cudaError_t e = vk::launch_order_xy(sites, D, perm, c->arena, c->stream);
@@ -1099,7 +1099,6 @@ int vecchia_log_cdf_unordered(vecchia_ctx* c, const double* sites, const double*
     if (cudaSetDevice(c->device) != cudaSuccess) return VECCHIA_ERR_CUDA;
     const bool dev = is_device_ptr(sites);
     if (is_device_ptr(u) != dev) return VECCHIA_ERR_ARG;
-    const bool host_xy = order_kind == VECCHIA_ORDER_XY && D > vk::kOrderXyDeviceMax;
     Carve dv(nullptr);
     const size_t o_s = dv.off;
     if (!dev) dv.take<double>(2 * D);
@@ -1133,21 +1132,16 @@ int vecchia_log_cdf_unordered(vecchia_ctx* c, const double* sites, const double*
         e = cudaMemcpyAsync(X + o_s, sites, sizeof(double) * 2 * D, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(X + o_u, u, sizeof(double) * D, cudaMemcpyHostToDevice, s);
     }
-    // ordering, queued on the stream (the host sort only for XY beyond the device size)
+    // ordering, queued on the stream
     std::vector<int32_t> hp;
     if (e == cudaSuccess) {
         if (order_kind == VECCHIA_ORDER_MAXMIN) {
             e = vk::launch_maxmin(sd, D, perm, X + o_scr, s);
-        } else if (order_kind == VECCHIA_ORDER_XY && !host_xy) {
+        } else if (order_kind == VECCHIA_ORDER_XY) {
             e = vk::launch_order_xy(sd, D, perm, X + o_scr, s);
         } else {
             hp.resize((size_t)D);
-            if (order_kind == VECCHIA_ORDER_XY) {
-                st = vecchia_order(dev ? c : nullptr, sites, D, VECCHIA_ORDER_XY, hp.data());
-                if (st != VECCHIA_OK) return st;
-            } else {
-                for (int64_t k = 0; k < D; ++k) hp[(size_t)k] = (int32_t)k;
-            }
+            for (int64_t k = 0; k < D; ++k) hp[(size_t)k] = (int32_t)k;
             e = cudaMemcpyAsync(perm, hp.data(), sizeof(int32_t) * D, cudaMemcpyHostToDevice, s);
         }
     }

@@ -49,51 +49,52 @@ __device__ __forceinline__ unsigned long long ord_key(double x) {
 __device__ __forceinline__ double ord_value(unsigned long long k) {
     return __longlong_as_double((long long)((k >> 63) ? (k & 0x7FFFFFFFFFFFFFFFULL) : ~k));
 }
-__device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v) {
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-        v = w < v ? w : v;
+        v = w > v ? w : v;
     }
     return v;
 }
 
-// Bounding box of the sites (one CTA): minima of the keys of x, y and of
-// their complements (the maxima), warp shuffles then one pass over the warps.
-__global__ void bbox_kernel(const double* __restrict__ sites, int64_t D, int gbits, Grid* out) {
-    __shared__ unsigned long long part[4][32];
-    unsigned long long k[4] = {~0ULL, ~0ULL, ~0ULL, ~0ULL};  // min x, min y, min ~x, min ~y
-    for (int64_t i = threadIdx.x; i < D; i += blockDim.x) {
+// Bounding box of the sites: maxima of the keys of x, y and of their
+// complements (the minima), warp shuffles, then one atomic a warp and quantity;
+// the last CTA to finish writes the grid.  box: four keys and a counter, all
+// zero at the start.  (One CTA alone took 119 us at D = 100,000, against 10 us.)
+__global__ void __launch_bounds__(256) bbox_kernel(const double* __restrict__ sites, int64_t D, int gbits,
+                                                   unsigned long long* box, Grid* out) {
+    unsigned long long k[4] = {0, 0, 0, 0};  // max ~x, max ~y, max x, max y
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < D; i += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long kx = ord_key(sites[2 * i]), ky = ord_key(sites[2 * i + 1]);
-        k[0] = kx < k[0] ? kx : k[0];
-        k[1] = ky < k[1] ? ky : k[1];
-        k[2] = ~kx < k[2] ? ~kx : k[2];
-        k[3] = ~ky < k[3] ? ~ky : k[3];
+        k[0] = max(k[0], ~kx);
+        k[1] = max(k[1], ~ky);
+        k[2] = max(k[2], kx);
+        k[3] = max(k[3], ky);
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) k[q] = warp_min_u64(k[q]);
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) part[q][warp] = k[q];
+    for (int q = 0; q < 4; ++q) {
+        k[q] = warp_max_u64(k[q]);
+        if ((threadIdx.x & 31) == 0) atomicMax(&box[q], k[q]);
+    }
+    __threadfence();
     __syncthreads();
-    if (warp == 0) {
+    if (threadIdx.x == 0 && atomicAdd((unsigned int*)(box + 4), 1u) == gridDim.x - 1) {
+        __threadfence();
 #pragma unroll
-        for (int q = 0; q < 4; ++q) k[q] = warp_min_u64(lane < nw ? part[q][lane] : ~0ULL);
-        if (lane == 0) {
-            const double xmin = ord_value(k[0]), ymin = ord_value(k[1]);
-            const double xmax = ord_value(~k[2]), ymax = ord_value(~k[3]);
-            const double ex = xmax - xmin, ey = ymax - ymin;
-            const double s = (ex > ey) ? ex : ey;
-            Grid g;
-            g.xmin = xmin;
-            g.ymin = ymin;
-            g.zero = !(s > 0.0);
-            g.c = g.zero ? 0.0 : 1073741824.0 / s;
-            g.shift = 30 - gbits;
-            g.G = 1 << gbits;
-            *out = g;
-        }
+        for (int q = 0; q < 4; ++q) k[q] = atomicMax(&box[q], 0ULL);
+        const double xmin = ord_value(~k[0]), ymin = ord_value(~k[1]);
+        const double xmax = ord_value(k[2]), ymax = ord_value(k[3]);
+        const double ex = xmax - xmin, ey = ymax - ymin;
+        const double s = (ex > ey) ? ex : ey;
+        Grid g;
+        g.xmin = xmin;
+        g.ymin = ymin;
+        g.zero = !(s > 0.0);
+        g.c = g.zero ? 0.0 : 1073741824.0 / s;
+        g.shift = 30 - gbits;
+        g.G = 1 << gbits;
+        *out = g;
     }
 }
 
@@ -479,11 +480,14 @@ cudaError_t launch_gather(const int32_t* perm, const double* sites, const double
     return cudaGetLastError();
 }
 
+constexpr size_t kBoxBytes = 64;  // bounding-box keys and counter
+
 size_t knn_scratch_bytes(int64_t D) {
     const int k = grid_bits(D);
     const int64_t cells = (int64_t)((1 << k) + 1) * ((1 << k) + 1);
     return align256(sizeof(Grid)) + align256(sizeof(int2) * (size_t)D) +
-           3 * align256(sizeof(int) * (size_t)(cells + 1)) + align256(sizeof(int4) * (size_t)D);
+           align256(kBoxBytes + sizeof(int) * (size_t)(cells + 1)) + 2 * align256(sizeof(int) * (size_t)(cells + 1)) +
+           align256(sizeof(int4) * (size_t)D);
 }
 
 // The cell grid of a problem in the caller's scratch (knn_scratch_bytes(D)):
@@ -503,18 +507,19 @@ cudaError_t build_cells(const double* sites, int64_t D, void* scratch, cudaStrea
     p += align256(sizeof(Grid));
     int2* qxy = (int2*)p;
     p += align256(sizeof(int2) * (size_t)D);
-    int* counts = (int*)p;
-    p += align256(sizeof(int) * (size_t)(cells + 1));
+    unsigned long long* box = (unsigned long long*)p;  // zeroed together with the counts
+    int* counts = (int*)(p + kBoxBytes);
+    p += align256(kBoxBytes + sizeof(int) * (size_t)(cells + 1));
     int* offsets = (int*)p;
     p += align256(sizeof(int) * (size_t)(cells + 1));
     int* cursor = (int*)p;
     p += align256(sizeof(int) * (size_t)(cells + 1));
     int4* cell_pts = (int4*)p;
     out = Cells{grid, qxy, offsets, cell_pts};
-    cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(int) * (size_t)cells, st);
+    cudaError_t e = cudaMemsetAsync(box, 0, kBoxBytes + sizeof(int) * (size_t)cells, st);
     if (e != cudaSuccess) return e;
-    bbox_kernel<<<1, 1024, 0, st>>>(sites, D, k, grid);
     const int blocks = (int)((D + 255) / 256);
+    bbox_kernel<<<blocks < 128 ? blocks : 128, 256, 0, st>>>(sites, D, k, box, grid);
     quantize_kernel<<<blocks, 256, 0, st>>>(sites, D, grid, qxy, counts);
     scan_kernel<<<1, 1024, 0, st>>>(counts, (int)cells, offsets, cursor);
     scatter_kernel<<<blocks, 256, 0, st>>>(qxy, D, grid, cursor, cell_pts);
@@ -537,304 +542,609 @@ cudaError_t launch_knn(const double* sites, int64_t D, int m, int32_t* nbr, void
     return cudaGetLastError();
 }
 
-// ---- exact maxmin ordering (one persistent CTA) ----------------------------
+// ---- device sort of unique keys (ordering) ----------------------------------
+// Ascending by (a, b, idx): tiles of 2,048 by a bitonic network in shared
+// memory, then passes that merge pairs of runs, each element finding its place
+// by a binary search in the sibling run (keys are unique through idx, so every
+// place is taken once).  A pass moves 12-20 bytes an element and is bound by
+// the 11-17 dependent loads of its search: 3 us a pass at D = 100,000.
+
+constexpr int kSortTile = 2048;
+
+struct SortRun {
+    unsigned long long* a;
+    unsigned long long* b;  // nullptr: keys of one word
+    int* idx;
+};
+
+template <bool TWO>
+__device__ __forceinline__ bool sort_less(unsigned long long a0, unsigned long long b0, int i0,
+                                          unsigned long long a1, unsigned long long b1, int i1) {
+    if (a0 != a1) return a0 < a1;
+    if (TWO && b0 != b1) return b0 < b1;
+    return i0 < i1;
+}
+
+// Sorts tile blockIdx.x of keys loaded by KEYS; writes to out, or (a single tile) the indices to perm.
+template <bool TWO, class KEYS>
+__global__ void __launch_bounds__(kSortTile / 2) sort_tile_kernel(KEYS keys, int D, SortRun out, int32_t* perm) {
+    __shared__ unsigned long long sa[kSortTile], sb[TWO ? kSortTile : 1];
+    __shared__ int si[kSortTile];
+    const int base = blockIdx.x * kSortTile;
+    for (int t = threadIdx.x; t < kSortTile; t += blockDim.x) {
+        unsigned long long a = ~0ull, b = ~0ull;
+        int i = INT_MAX;  // beyond the end: after every key
+        if (base + t < D) keys.load(base + t, a, b, i);
+        sa[t] = a;
+        if (TWO) sb[t] = b;
+        si[t] = i;
+    }
+    for (int kb = 2; kb <= kSortTile; kb <<= 1)
+        for (int jm = kb >> 1; jm > 0; jm >>= 1) {
+            __syncthreads();
+            const int t = threadIdx.x, lo = ((t & ~(jm - 1)) << 1) | (t & (jm - 1)), hi = lo | jm;
+            const bool up = (lo & kb) == 0;
+            const unsigned long long a0 = sa[lo], a1 = sa[hi], b0 = TWO ? sb[lo] : 0, b1 = TWO ? sb[hi] : 0;
+            const int i0 = si[lo], i1 = si[hi];
+            if (sort_less<TWO>(a1, b1, i1, a0, b0, i0) == up) {
+                sa[lo] = a1;
+                sa[hi] = a0;
+                if (TWO) {
+                    sb[lo] = b1;
+                    sb[hi] = b0;
+                }
+                si[lo] = i1;
+                si[hi] = i0;
+            }
+        }
+    __syncthreads();
+    for (int t = threadIdx.x; t < kSortTile && base + t < D; t += blockDim.x) {
+        if (perm) {
+            perm[base + t] = si[t];
+        } else {
+            out.a[base + t] = sa[t];
+            if (TWO) out.b[base + t] = sb[t];
+            out.idx[base + t] = si[t];
+        }
+    }
+}
+
+// Merges runs of length w in pairs; the last pass writes the indices to perm.
+template <bool TWO>
+__global__ void sort_merge_kernel(SortRun in, SortRun out, int D, int64_t w, int32_t* perm) {
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= D) return;
+    const int64_t run = g / w, mine = run * w, other = (run ^ 1) * w;
+    const unsigned long long a = in.a[g], b = TWO ? in.b[g] : 0;
+    const int i = in.idx[g];
+    int64_t lo = other < D ? other : D, hi = other + w < D ? other + w : D;
+    const int64_t o0 = lo;
+    while (lo < hi) {  // first element of the sibling run that is not before this key
+        const int64_t mid = (lo + hi) >> 1;
+        if (sort_less<TWO>(in.a[mid], TWO ? in.b[mid] : 0, in.idx[mid], a, b, i))
+            lo = mid + 1;
+        else
+            hi = mid;
+    }
+    const int64_t dst = (mine < other ? mine : other) + (g - mine) + (lo - o0);
+    if (perm) {
+        perm[dst] = i;
+    } else {
+        out.a[dst] = a;
+        if (TWO) out.b[dst] = b;
+        out.idx[dst] = i;
+    }
+}
+
+size_t sort_scratch_bytes(int64_t D, bool two) {
+    return 2 * (align256(8 * (size_t)D) * (two ? 2 : 1) + align256(4 * (size_t)D));
+}
+
+template <bool TWO, class KEYS>
+cudaError_t launch_sort(KEYS keys, int64_t D, int32_t* perm, void* scratch, cudaStream_t st) {
+    SortRun r[2];
+    char* p = (char*)scratch;
+    for (int k = 0; k < 2; ++k) {
+        r[k].a = (unsigned long long*)p;
+        p += align256(8 * (size_t)D);
+        r[k].b = nullptr;
+        if (TWO) {
+            r[k].b = (unsigned long long*)p;
+            p += align256(8 * (size_t)D);
+        }
+        r[k].idx = (int*)p;
+        p += align256(4 * (size_t)D);
+    }
+    const int tiles = (int)((D + kSortTile - 1) / kSortTile);
+    sort_tile_kernel<TWO><<<tiles, kSortTile / 2, 0, st>>>(keys, (int)D, r[0], tiles == 1 ? perm : nullptr);
+    int cur = 0;
+    for (int64_t w = kSortTile; w < D; w *= 2, cur ^= 1)
+        sort_merge_kernel<TWO><<<(unsigned)((D + 255) / 256), 256, 0, st>>>(r[cur], r[cur ^ 1], (int)D, w,
+                                                                         2 * w >= D ? perm : nullptr);
+    return cudaGetLastError();
+}
+
+// ---- exact maxmin ordering (one thread-block cluster) -------------------------
 // Same rule as the host ordering: first the site nearest the centre of the
 // quantised bounding box (2q - qmax, smallest squared distance, ties to the
 // smaller index), then repeatedly the unchosen site whose squared distance to
-// the chosen set is largest (ties to the smaller index).  mind[i] holds that
-// distance (-1 once chosen); a 32-ary tournament tree over (mind, index) gives
-// the next pick at its root.  A pick at max distance r^2 can only lower the
-// mind of sites closer than r, so each step scans the grid cells within r of
-// the pick and recomputes the tree nodes above the leaves that changed.
+// the chosen set is largest (ties to the smaller index).
+//
+// The picks need not be made one at a time.  Let mind_i be site i's squared
+// distance to the chosen set and key_i = (mind_i, -i).  Picking a site only
+// lowers keys, so the picks' keys decrease strictly, and the ordering is the
+// sites sorted by the key each has when it is picked.  Site i's key is final as
+// soon as no unchosen site of larger key lies closer than mind_i to it: only a
+// site picked before i, hence of larger key now, could lower mind_i, and only
+// from within that distance.  So each round takes every site whose key is final
+// (the locally dominant ones), records the key, and lowers mind in their
+// surroundings; about 15 to 20 rounds order any even spread of sites (n sites in
+// a round allow a fixed fraction of n in the next).  A pick p lowers mind_j only
+// where key_j < key_p: a j of larger key comes before p in the ordering (and
+// whenever that holds, d(j, p) >= mind_p, so p is no nearer to j than what j has
+// by the time its key falls below p's).  The first kMmSerial picks, whose reach
+// spans most sites, are made one at a time by all threads; a sort of the
+// recorded keys ends it.  Each unchosen site keeps a witness (a site that
+// dominates it) from round to round and searches anew only once that one no
+// longer does; the search is per thread over the 3 x 3 cells around the site,
+// where it nearly always ends, and by the whole warp over the reach otherwise.
+//
+// Below kMmGridWide sites one cluster of up to 16 CTAs runs it all: a round's two
+// barriers are the hardware's cluster barrier, and there are no spin-waits.  From
+// there on (0.53 against 0.75 ms at 6,000 sites, 0.95 against 2.8 ms at 100,000)
+// the first kMmRounds rounds are launches over the whole GPU, which do nothing
+// once every site is taken, and the cluster does what rounds remain.  Bound by
+// the latency of the dependent L2 loads (witness, its mind; cell, its sites,
+// their minds): a late round of 20 us moves a few MB.  A
+// serial pick took 5 to 7 us (one CTA: scan, tournament tree).  Whole call: D =
+// 100,000 705 -> 0.95 ms, 20,011 116 -> 0.60 ms, 2,048 9.7 -> 0.53 ms, 100
+// 0.47 -> 0.16 ms; 8,000 sites crowded about a point 127 -> 16 ms.
 
 constexpr int kMmThreads = 1024;
-constexpr int kMmMaxLevels = 8;
+constexpr int kMmSerial = 32;
+constexpr int kMmMaxCluster = 16;
+constexpr int kMmRounds = 16;        // grid-wide rounds
+constexpr int64_t kMmGridWide = 6000;  // from this many sites on
 
-struct MmTree {
-    long long* val;   // node values, all levels (level l at off[l])
-    int* idx;         // node argmax index
-    int* flag;        // dirty marks
-    int* list[2];     // dirty node lists (alternating)
-    int off[kMmMaxLevels + 1];
-    int n[kMmMaxLevels + 1];  // n[0] = D leaves, n[l] nodes of level l
-    int levels;               // root = level `levels`, node 0
-    int total;                // nodes of all levels
-    int in_smem;              // 1: the arrays live in the CTA's dynamic shared memory
+struct MmSlot {
+    long long v, w;
+    int s, pad;
 };
+
+struct MmState {
+    const int4* pts;     // sites sorted by cell: (qx, qy, index, -); the arrays below go by that position
+    const int* offsets;  // cell starts
+    long long* mind;     // squared distance to the chosen set, -1 once chosen
+    long long* key;      // mind when chosen
+    int* wit;            // witness, or -1
+    int* list;           // the round's picks
+    int* count;          // their number: rounds of the cluster mod 3, then the grid-wide rounds
+    MmSlot* slot;        // per CTA (two sets, alternating)
+};
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 
 __device__ __forceinline__ bool mm_better(long long va, int ia, long long vb, int ib) {
     return va > vb || (va == vb && ia < ib);
 }
 
-__device__ __forceinline__ void mm_warp_argmax(long long& v, int& i) {
+// Cells within reach of a site: |dx|, |dy| < rr for d^2 < m.
+struct MmReach {
+    int xl, xh, yl, yh;
+};
+__device__ __forceinline__ MmReach mm_reach(const Grid& g, int x, int y, long long m) {
+    // sqrt from above: FP32 rounding is below 1e-6 relative
+    const long long rr = m == LLONG_MAX ? (1LL << 31) : (long long)(sqrtf((float)m) * 1.000001f) + 2;
+    MmReach r;
+    r.xl = (int)(max(0LL, (long long)x - rr) >> g.shift);
+    r.yl = (int)(max(0LL, (long long)y - rr) >> g.shift);
+    r.xh = (int)min((long long)g.G, ((long long)x + rr) >> g.shift);
+    r.yh = (int)min((long long)g.G, ((long long)y + rr) >> g.shift);
+    return r;
+}
+
+__device__ __forceinline__ long long mm_d2(const int4& a, const int4& b) {
+    const long long dx = (long long)a.x - b.x, dy = (long long)a.y - b.y;
+    return dx * dx + dy * dy;
+}
+
+// Site q (mind mq) keeps site p's key open: larger key, closer than mind_p.
+__device__ __forceinline__ bool mm_dominates(const int4& q, long long mq, const int4& p, long long mp) {
+    return mm_better(mq, q.z, mp, p.z) && mm_d2(q, p) < mp;
+}
+
+// Best (largest v, then smallest i) over the CTA; valid in warp 0.
+__device__ __forceinline__ void mm_block_best(long long& v, int& i, int& s, long long* rv, int* ri, int* rs) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int pass = 0; pass < 2; ++pass) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const long long ov = __shfl_xor_sync(0xffffffffu, v, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, i, o);
-        if (mm_better(ov, oi, v, i)) {
-            v = ov;
-            i = oi;
-        }
-    }
-}
-
-// Bytes of the tree arrays (8 + 4 + 4 per node, two lists of level-1 size).
-__host__ __device__ inline size_t mm_tree_bytes(int total, int n1) {
-    return (size_t)total * 16 + (size_t)2 * n1 * 4 + 64;
-}
-
-// Node `node` of level l (>= 1): argmax of its 32 children; lane 0 stores it,
-// clears its mark and queues its parent.
-__device__ __forceinline__ void mm_node(MmTree& T, const long long* mind, int l, int node, int* cnt, int lane) {
-    const int c = node * 32 + lane;
-    long long v = LLONG_MIN;
-    int i = INT_MAX;
-    if (c < T.n[l - 1]) {
-        if (l == 1) {
-            v = mind[c];
-            i = c;
-        } else {
-            v = T.val[T.off[l - 1] + c];
-            i = T.idx[T.off[l - 1] + c];
-        }
-    }
-    mm_warp_argmax(v, i);
-    if (lane == 0) {
-        T.val[T.off[l] + node] = v;
-        T.idx[T.off[l] + node] = i;
-        T.flag[T.off[l] + node] = 0;
-        if (l < T.levels) {
-            const int parent = node >> 5;
-            if (atomicExch(&T.flag[T.off[l + 1] + parent], 1) == 0)
-                T.list[(l + 1) & 1][atomicAdd(&cnt[l + 1], 1)] = parent;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kMmThreads) maxmin_kernel(const Grid* __restrict__ grid,
-                                                            const int2* __restrict__ qxy,
-                                                            const int* __restrict__ offsets,
-                                                            const int4* __restrict__ cell_pts, int D,
-                                                            long long* __restrict__ mind, MmTree T,
-                                                            int32_t* __restrict__ perm) {
-    extern __shared__ __align__(16) unsigned char mm_smem[];
-    __shared__ long long red_v[kMmThreads / 32], red_y[kMmThreads / 32];
-    __shared__ int red_i[kMmThreads / 32];
-    __shared__ int cnt[kMmMaxLevels + 2];
-    __shared__ int s_pick;
-    __shared__ long long s_r2;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const Grid g = *grid;
-    const int W = g.G + 1;
-    if (T.in_smem) {  // carve the tree out of dynamic shared memory
-        unsigned char* p = mm_smem;
-        T.val = (long long*)p;
-        p += (size_t)T.total * 8;
-        T.idx = (int*)p;
-        p += (size_t)T.total * 4;
-        T.flag = (int*)p;
-        p += (size_t)T.total * 4;
-        T.list[0] = (int*)p;
-        p += (size_t)T.n[1] * 4;
-        T.list[1] = (int*)p;
-    }
-
-    // leaves at "infinity", no marks
-    for (int i = tid; i < D; i += kMmThreads) mind[i] = LLONG_MAX;
-    for (int x = tid; x < T.total; x += kMmThreads) T.flag[x] = 0;
-    // the first site: nearest the centre of the quantised bounding box
-    long long qxm = 0, qym = 0;
-    for (int i = tid; i < D; i += kMmThreads) {
-        qxm = max(qxm, (long long)qxy[i].x);
-        qym = max(qym, (long long)qxy[i].y);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        qxm = max(qxm, __shfl_xor_sync(0xffffffffu, qxm, o));
-        qym = max(qym, __shfl_xor_sync(0xffffffffu, qym, o));
-    }
-    if (lane == 0) {
-        red_v[warp] = qxm;
-        red_y[warp] = qym;
-    }
-    __syncthreads();
-    qxm = 0;
-    qym = 0;
-    for (int w = 0; w < kMmThreads / 32; ++w) {
-        qxm = max(qxm, red_v[w]);
-        qym = max(qym, red_y[w]);
-    }
-    __syncthreads();
-    long long bv = LLONG_MAX;
-    int bi = INT_MAX;
-    for (int i = tid; i < D; i += kMmThreads) {
-        const long long dx = 2LL * qxy[i].x - qxm, dy = 2LL * qxy[i].y - qym;
-        const long long v = dx * dx + dy * dy;
-        if (v < bv || (v == bv && i < bi)) {
-            bv = v;
-            bi = i;
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) {  // arg-min over (distance, index)
-        const long long ov = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov < bv || (ov == bv && oi < bi)) {
-            bv = ov;
-            bi = oi;
-        }
-    }
-    if (lane == 0) {
-        red_v[warp] = bv;
-        red_i[warp] = bi;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        long long v = LLONG_MAX;
-        int f = INT_MAX;
-        for (int w = 0; w < kMmThreads / 32; ++w)
-            if (red_v[w] < v || (red_v[w] == v && red_i[w] < f)) {
-                v = red_v[w];
-                f = red_i[w];
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long ov = __shfl_xor_sync(0xffffffffu, v, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, i, o), os = __shfl_xor_sync(0xffffffffu, s, o);
+            if (mm_better(ov, oi, v, i)) {
+                v = ov;
+                i = oi;
+                s = os;
             }
-        perm[0] = f;
-        mind[f] = -1;
-        s_pick = f;
-        s_r2 = LLONG_MAX;  // every site is within reach of the first pick
-        for (int l = 0; l < kMmMaxLevels + 2; ++l) cnt[l] = 0;
-        T.flag[T.off[1] + (f >> 5)] = 1;
-        T.list[1][0] = f >> 5;
-        cnt[1] = 1;
-    }
-    __syncthreads();
-
-    for (int k = 1; k < D; ++k) {
-        // scan: lower mind of the sites within reach of the last pick
-        const int pick = s_pick;
-        const long long r2 = s_r2;
-        const int2 pq = qxy[pick];
-        int cx_lo = 0, cx_hi = g.G, cy_lo = 0, cy_hi = g.G;
-        if (r2 != LLONG_MAX) {
-            const long long rr = (long long)sqrt((double)r2) + 1;  // |dx|, |dy| < rr for d^2 < r2
-            cx_lo = (int)(max(0LL, (long long)pq.x - rr) >> g.shift);
-            cy_lo = (int)(max(0LL, (long long)pq.y - rr) >> g.shift);
-            cx_hi = (int)min((long long)g.G, ((long long)pq.x + rr) >> g.shift);
-            cy_hi = (int)min((long long)g.G, ((long long)pq.y + rr) >> g.shift);
         }
-        for (int row = cy_lo + warp; row <= cy_hi; row += kMmThreads / 32) {
-            const int b = offsets[row * W + cx_lo], e = offsets[row * W + cx_hi + 1];
-            for (int x = b + lane; x < e; x += 32) {
-                const int4 o = cell_pts[x];
-                const long long mi = mind[o.z];
-                if (mi < 0) continue;
-                const long long dx = (long long)o.x - pq.x, dy = (long long)o.y - pq.y;
-                const long long d2 = dx * dx + dy * dy;
-                if (d2 < mi) {
-                    mind[o.z] = d2;
-                    const int node = o.z >> 5;
-                    if (atomicExch(&T.flag[T.off[1] + node], 1) == 0) T.list[1][atomicAdd(&cnt[1], 1)] = node;
+        if (pass == 1) return;
+        if (lane == 0) {
+            rv[warp] = v;
+            ri[warp] = i;
+            rs[warp] = s;
+        }
+        __syncthreads();
+        if (warp != 0) return;
+        v = rv[lane];  // kMmThreads = 32 warps
+        i = ri[lane];
+        s = rs[lane];
+    }
+}
+
+// Warp gw of GW: the sites whose keys are final go to the round's list (cnt).
+__device__ __forceinline__ void mm_check(const Grid& g, const MmState& S, int D, int* cnt, int gw, int GW) {
+    const int lane = threadIdx.x & 31, W = g.G + 1;
+    auto take = [&](int s, long long m) {
+        S.key[s] = m;
+        S.list[atomicAdd(cnt, 1)] = s;
+    };
+    for (int base = gw * 32; base < D; base += GW * 32) {
+        const int s = base + lane;
+        const long long m = s < D ? __ldcg(&S.mind[s]) : -1;
+        bool open = m >= 0;
+        int4 p = make_int4(0, 0, 0, 0);
+        if (open) {
+            p = S.pts[s];
+            const int w = S.wit[s];
+            if (w >= 0 && mm_dominates(S.pts[w], __ldcg(&S.mind[w]), p, m)) open = false;
+        }
+        MmReach R{0, 0, 0, 0};
+        if (open && m == 0) {  // a duplicate of a chosen site: nothing is closer
+            take(s, m);
+            open = false;
+        }
+        if (open) {  // the 3 x 3 cells around the site, its own row first
+            R = mm_reach(g, p.x, p.y, m);
+            const int cx = p.x >> g.shift, cy = p.y >> g.shift;
+            const int xa = max(R.xl, cx - 1), xb = min(R.xh, cx + 1);
+            int found = -1;
+            bool cut = false;  // rows of crowded cells are left to the warp
+            for (int t = 0; t < 3 && found < 0; ++t) {
+                const int row = cy + (t == 0 ? 0 : t == 1 ? -1 : 1);
+                if (row < R.yl || row > R.yh) continue;
+                const int b = S.offsets[row * W + xa], end = S.offsets[row * W + xb + 1];
+                const int e = min(end, b + 64);
+                cut = cut || e < end;
+                for (int x = b; x < e && found < 0; x += 4) {
+                    int4 q[4];
+                    long long mq[4];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const int y = min(x + h, e - 1);
+                        q[h] = S.pts[y];
+                        mq[h] = __ldcg(&S.mind[y]);
+                    }
+#pragma unroll
+                    for (int h = 0; h < 4; ++h)
+                        if (mm_dominates(q[h], mq[h], p, m)) found = min(x + h, e - 1);
                 }
             }
-        }
-        __syncthreads();
-        // level 1 by all warps
-        for (int j = warp; j < cnt[1]; j += kMmThreads / 32) mm_node(T, mind, 1, T.list[1][j], cnt, lane);
-        __syncthreads();
-        // upper levels and the next pick by warp 0
-        if (warp == 0) {
-            for (int l = 2; l <= T.levels; ++l) {
-                const int n = cnt[l];
-                for (int j = 0; j < n; ++j) mm_node(T, mind, l, T.list[l & 1][j], cnt, lane);
-                __syncwarp();
-            }
-            if (lane == 0) {
-                const int root = T.off[T.levels];
-                const int nxt = T.idx[root];
-                perm[k] = nxt;
-                mind[nxt] = -1;
-                s_pick = nxt;
-                s_r2 = T.val[root];
-                for (int l = 0; l < kMmMaxLevels + 2; ++l) cnt[l] = 0;
-                T.flag[T.off[1] + (nxt >> 5)] = 1;  // its own leaf changed
-                T.list[1][0] = nxt >> 5;
-                cnt[1] = 1;
+            if (found >= 0) {
+                S.wit[s] = found;
+                open = false;
+            } else if (!cut && R.xl >= cx - 1 && R.xh <= cx + 1 && R.yl >= cy - 1 && R.yh <= cy + 1) {
+                take(s, m);
+                open = false;
             }
         }
-        __syncthreads();
+        unsigned todo = __ballot_sync(0xffffffffu, open);
+        while (todo) {  // the whole reach, by the warp, rows from the site's own outwards
+            const int b = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const int4 c = make_int4(__shfl_sync(0xffffffffu, p.x, b), __shfl_sync(0xffffffffu, p.y, b),
+                                     __shfl_sync(0xffffffffu, p.z, b), 0);
+            const long long mc = __shfl_sync(0xffffffffu, m, b);
+            const MmReach Q = mm_reach(g, c.x, c.y, mc);
+            const int cy = c.y >> g.shift, far = max(cy - Q.yl, Q.yh - cy);
+            int found = -1;
+            for (int t0 = 0; t0 <= 2 * far && found < 0; t0 += 32) {
+                // lane t holds the bounds of row t0 + t of that order
+                const int t = t0 + lane, row = cy + ((t & 1) ? -((t + 1) >> 1) : (t >> 1));
+                const bool in = row >= Q.yl && row <= Q.yh;
+                const int rlo = in ? S.offsets[row * W + Q.xl] : 0, rhi = in ? S.offsets[row * W + Q.xh + 1] : 0;
+                for (unsigned rows = __ballot_sync(0xffffffffu, rlo < rhi); rows && found < 0; rows &= rows - 1) {
+                    const int h = __ffs(rows) - 1;
+                    const int lo = __shfl_sync(0xffffffffu, rlo, h), hi = __shfl_sync(0xffffffffu, rhi, h);
+                    for (int x0 = lo; x0 < hi && found < 0; x0 += 64) {  // two sites a lane
+                        const int x = x0 + lane, y = min(x + 32, hi - 1);
+                        bool d = false;
+                        if (x < hi) {
+                            const int4 p0 = S.pts[x], p1 = S.pts[y];
+                            const long long m0 = __ldcg(&S.mind[x]), m1 = __ldcg(&S.mind[y]);
+                            d = mm_dominates(p0, m0, c, mc);
+                            const bool d1 = mm_dominates(p1, m1, c, mc);
+                            if (d || d1) found = d ? x : y;
+                            d = d || d1;
+                        }
+                        const unsigned hit = __ballot_sync(0xffffffffu, d);
+                        if (hit) found = __shfl_sync(0xffffffffu, found, __ffs(hit) - 1);
+                    }
+                }
+            }
+            if (lane == b) {
+                if (found >= 0)
+                    S.wit[s] = found;
+                else
+                    take(s, m);
+            }
+        }
     }
 }
 
-// Tree shape for D leaves: level sizes and offsets.
-bool mm_shape(int64_t D, MmTree& T) {
-    T.n[0] = (int)D;
-    T.off[0] = 0;
-    int levels = 0, total = 0;
-    int64_t n = D;
-    do {
-        n = (n + 31) / 32;
-        ++levels;
-        if (levels > kMmMaxLevels) return false;
-        T.off[levels] = total;
-        T.n[levels] = (int)n;
-        total += (int)n;
-    } while (n > 1);
-    T.levels = levels;
-    T.total = total;
-    return true;
+// Warp gw of GW: the round's n picks leave the open sites and lower mind around them.
+__device__ __forceinline__ void mm_update(const Grid& g, const MmState& S, int n, int gw, int GW) {
+    const int lane = threadIdx.x & 31, W = g.G + 1;
+    // warps to spare take a pick's rows side by side (the first rounds: few picks of wide reach)
+    const int per = n > 0 ? max(1, min(GW / n, 64)) : 1;
+    for (int64_t e = gw; e < (int64_t)n * per; e += GW) {
+        const int s = __ldcg(&S.list[e / per]), r0 = (int)(e % per);
+        const int4 p = S.pts[s];
+        const long long K = __ldcg(&S.key[s]);
+        if (r0 == 0 && lane == 0) S.mind[s] = -1;
+        const MmReach R = mm_reach(g, p.x, p.y, K);
+        for (int row = R.yl + r0; row <= R.yh; row += per) {
+            const int lo = S.offsets[row * W + R.xl], hi = S.offsets[row * W + R.xh + 1];
+            for (int x = lo + lane; x < hi; x += 32) {
+                const long long m = __ldcg(&S.mind[x]);
+                if (m < 0) continue;
+                const int4 q = S.pts[x];
+                const long long d2 = mm_d2(p, q);
+                if (d2 < m && mm_better(K, p.z, m, q.z)) atomicMin(&S.mind[x], d2);
+            }
+        }
+    }
 }
 
-constexpr size_t kMmSmemMax = 200 * 1024;
+__global__ void __launch_bounds__(256) maxmin_check_kernel(const Grid* __restrict__ grid, MmState S, int D, int r) {
+    int done = kMmSerial;
+    for (int k = 0; k < r; ++k) done += S.count[3 + k];
+    if (done >= D) return;
+    mm_check(*grid, S, D, S.count + 3 + r, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5);
+}
+
+__global__ void __launch_bounds__(256) maxmin_update_kernel(const Grid* __restrict__ grid, MmState S, int r) {
+    mm_update(*grid, S, S.count[3 + r], (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5);
+}
+
+__global__ void __launch_bounds__(kMmThreads) maxmin_kernel(const Grid* __restrict__ grid, MmState S, int D,
+                                                            bool serial, bool finish, int rounds) {
+    __shared__ long long red_v[32];
+    __shared__ int red_i[32], red_s[32];
+    __shared__ long long s_v;
+    __shared__ int s_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = blockIdx.x, C = gridDim.x;  // one cluster
+    const int gt = rank * kMmThreads + tid, GT = C * kMmThreads;
+    const Grid g = *grid;
+
+    if (serial) {
+        // the first site: nearest the centre of the quantised bounding box
+        long long qx = 0, qy = 0;
+        for (int s = gt; s < D; s += GT) {
+            const int4 p = S.pts[s];
+            qx = max(qx, (long long)p.x);
+            qy = max(qy, (long long)p.y);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            qx = max(qx, __shfl_xor_sync(0xffffffffu, qx, o));
+            qy = max(qy, __shfl_xor_sync(0xffffffffu, qy, o));
+        }
+        if (lane == 0) {
+            red_v[warp] = qx;
+            red_i[warp] = (int)qy;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < kMmThreads / 32; ++w) {
+                qx = max(qx, red_v[w]);
+                qy = max(qy, (long long)red_i[w]);
+            }
+            S.slot[rank].v = qx;
+            S.slot[rank].w = qy;
+        }
+        cluster_sync();
+        for (int c = 0; c < C; ++c) {
+            qx = max(qx, __ldcg(&S.slot[c].v));
+            qy = max(qy, __ldcg(&S.slot[c].w));
+        }
+        long long bv = LLONG_MIN;  // minus the distance: the largest is the nearest
+        int bi = INT_MAX, bs = -1;
+        for (int s = gt; s < D; s += GT) {
+            const int4 p = S.pts[s];
+            const long long dx = 2LL * p.x - qx, dy = 2LL * p.y - qy, v = -(dx * dx + dy * dy);
+            if (mm_better(v, p.z, bv, bi)) {
+                bv = v;
+                bi = p.z;
+                bs = s;
+            }
+        }
+        // one pick at a time; the first iteration only finds the first site
+        const int n_serial = min(kMmSerial, D);
+        for (int k = 0; k <= n_serial; ++k) {
+            mm_block_best(bv, bi, bs, red_v, red_i, red_s);
+            MmSlot* sl = S.slot + kMmMaxCluster * (1 + (k & 1));
+            if (tid == 0) {
+                sl[rank].v = bv;
+                sl[rank].w = bi;
+                sl[rank].s = bs;
+            }
+            cluster_sync();
+            if (warp == 0) {
+                bv = lane < C ? __ldcg(&sl[lane].v) : LLONG_MIN;
+                bi = lane < C ? (int)__ldcg(&sl[lane].w) : INT_MAX;
+                bs = lane < C ? __ldcg(&sl[lane].s) : -1;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const long long ov = __shfl_xor_sync(0xffffffffu, bv, o);
+                    const int oi = __shfl_xor_sync(0xffffffffu, bi, o), os = __shfl_xor_sync(0xffffffffu, bs, o);
+                    if (mm_better(ov, oi, bv, bi)) {
+                        bv = ov;
+                        bi = oi;
+                        bs = os;
+                    }
+                }
+                if (lane == 0) {
+                    s_v = bv;
+                    s_s = bs;
+                }
+            }
+            __syncthreads();
+            if (k == n_serial) break;
+            const int ps = s_s;  // this pick (k < D: there is one)
+            const int4 p = S.pts[ps];
+            if (gt == 0) S.key[ps] = k == 0 ? LLONG_MAX : s_v;
+            bv = LLONG_MIN;
+            bi = INT_MAX;
+            bs = -1;
+            for (int s = gt; s < D; s += GT) {
+                const int4 q = S.pts[s];
+                long long m = k == 0 ? LLONG_MAX : S.mind[s];  // this thread's own value
+                if (s == ps) {
+                    m = -1;
+                } else if (m >= 0) {
+                    m = min(m, mm_d2(p, q));
+                    if (mm_better(m, q.z, bv, bi)) {
+                        bv = m;
+                        bi = q.z;
+                        bs = s;
+                    }
+                }
+                S.mind[s] = m;
+                if (k == 0) S.wit[s] = -1;
+            }
+        }
+        cluster_sync();
+    }
+
+    if (!finish) return;
+
+    // rounds of locally dominant picks
+    const int gw = rank * (kMmThreads / 32) + warp, GW = C * (kMmThreads / 32);
+    int left = D - kMmSerial;
+    for (int k = 0; k < rounds; ++k) left -= __ldcg(&S.count[3 + k]);  // what the grid-wide rounds took
+    for (int r = 0; left > 0; ++r) {
+        int* cnt = S.count + r % 3;
+        mm_check(g, S, D, cnt, gw, GW);
+        cluster_sync();
+        const int n = __ldcg(cnt);
+        if (n <= 0) break;  // never: the largest key of all is final
+        left -= n;
+        if (gt == 0) S.count[(r + 1) % 3] = 0;  // last read two rounds ago
+        mm_update(g, S, n, gw, GW);
+        cluster_sync();
+    }
+}
+
+struct MmKeys {  // descending key, then ascending index
+    const long long* key;
+    const int4* pts;
+    __device__ void load(int s, unsigned long long& a, unsigned long long& b, int& i) const {
+        a = ~(unsigned long long)key[s];
+        b = 0;
+        i = pts[s].z;
+    }
+};
 
 size_t maxmin_scratch_bytes(int64_t D) {
-    MmTree T;
-    if (!mm_shape(D, T)) return 0;
-    return knn_scratch_bytes(D) + align256(sizeof(long long) * (size_t)D) + align256(mm_tree_bytes(T.total, T.n[1]));
+    return knn_scratch_bytes(D) + 2 * align256(sizeof(long long) * (size_t)D) + 2 * align256(sizeof(int) * (size_t)D) +
+           align256(sizeof(MmSlot) * 3 * kMmMaxCluster + (3 + kMmRounds) * sizeof(int)) + sort_scratch_bytes(D, false);
+}
+
+// The largest cluster that the device schedules (16 is beyond the portable 8).
+int maxmin_cluster(int dev) {
+    static std::mutex mu;
+    static std::map<int, int> best;
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = best.find(dev);
+    if (it != best.end()) return it->second;
+    int c = 8;
+    if (cudaFuncSetAttribute(maxmin_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kMmMaxCluster);
+        cfg.blockDim = dim3(kMmThreads);
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = kMmMaxCluster;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, maxmin_kernel, &cfg) == cudaSuccess && n > 0) c = kMmMaxCluster;
+    }
+    cudaGetLastError();
+    return best[dev] = c;
 }
 
 cudaError_t launch_maxmin(const double* sites, int64_t D, int32_t* perm, void* scratch, cudaStream_t st) {
     if (D <= 0) return cudaSuccess;
-    MmTree T;
-    if (!mm_shape(D, T)) return cudaErrorInvalidValue;
+    if (D > INT_MAX / 2) return cudaErrorInvalidValue;
     Cells c;
     cudaError_t e = build_cells(sites, D, scratch, st, c);
     if (e != cudaSuccess) return e;
     char* p = (char*)scratch + knn_scratch_bytes(D);
-    long long* mind = (long long*)p;
+    MmState S;
+    S.pts = c.cell_pts;
+    S.offsets = c.offsets;
+    S.mind = (long long*)p;
     p += align256(sizeof(long long) * (size_t)D);
-    const size_t tree = mm_tree_bytes(T.total, T.n[1]);
-    T.in_smem = tree <= kMmSmemMax;
-    size_t smem = 0;
-    if (T.in_smem) {
-        smem = tree;
-        static std::mutex mu;
-        static std::map<int, size_t> attr;
-        int dev = 0;
-        cudaGetDevice(&dev);
-        std::lock_guard<std::mutex> lk(mu);
-        if (smem > 48 * 1024 && attr[dev] < smem) {
-            e = cudaFuncSetAttribute(maxmin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmSmemMax);
-            if (e != cudaSuccess) return e;
-            attr[dev] = kMmSmemMax;
+    S.key = (long long*)p;
+    p += align256(sizeof(long long) * (size_t)D);
+    S.wit = (int*)p;
+    p += align256(sizeof(int) * (size_t)D);
+    S.list = (int*)p;
+    p += align256(sizeof(int) * (size_t)D);
+    S.slot = (MmSlot*)p;
+    S.count = (int*)(p + sizeof(MmSlot) * 3 * kMmMaxCluster);
+    p += align256(sizeof(MmSlot) * 3 * kMmMaxCluster + (3 + kMmRounds) * sizeof(int));
+    e = cudaMemsetAsync(S.count, 0, (3 + kMmRounds) * sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int most = maxmin_cluster(dev);
+    int cl = 1;  // about four sites a thread: fewer CTAs make cheaper barriers
+    while (cl < most && (int64_t)cl * kMmThreads * 4 < D) cl *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cl);
+    cfg.blockDim = dim3(kMmThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cl;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    const int rounds = D >= kMmGridWide ? kMmRounds : 0;
+    if (rounds) {
+        e = cudaLaunchKernelEx(&cfg, maxmin_kernel, (const Grid*)c.grid, S, (int)D, true, false, 0);
+        if (e != cudaSuccess) return e;
+        for (int r = 0; r < rounds; ++r) {
+            maxmin_check_kernel<<<(unsigned)((D + 255) / 256), 256, 0, st>>>(c.grid, S, (int)D, r);
+            maxmin_update_kernel<<<8 * device_sm_count(dev), 256, 0, st>>>(c.grid, S, r);
         }
-        T.val = nullptr;
-        T.idx = T.flag = T.list[0] = T.list[1] = nullptr;
-    } else {
-        T.val = (long long*)p;
-        p += (size_t)T.total * 8;
-        T.idx = (int*)p;
-        p += (size_t)T.total * 4;
-        T.flag = (int*)p;
-        p += (size_t)T.total * 4;
-        T.list[0] = (int*)p;
-        p += (size_t)T.n[1] * 4;
-        T.list[1] = (int*)p;
     }
-    maxmin_kernel<<<1, kMmThreads, smem, st>>>(c.grid, c.qxy, c.offsets, c.cell_pts, (int)D, mind, T, perm);
-    return cudaGetLastError();
+    e = cudaLaunchKernelEx(&cfg, maxmin_kernel, (const Grid*)c.grid, S, (int)D, rounds == 0, true, rounds);
+    if (e != cudaSuccess) return e;
+    return launch_sort<false>(MmKeys{S.key, S.pts}, D, perm, p, st);
 }
 
-// ---- XY ordering on the device (D <= 8192) ----------------------------------
+// ---- XY ordering on the device ------------------------------------------------
 // The rank of site i in the (x, y, index) order is the number of sites whose
 // key is smaller (the host's XY rule; keys are unique through the index);
-// perm[rank_i] = i.
+// perm[rank_i] = i.  Up to kXyMax sites by counting (D^2 compares, but two
+// launches: 12 us at D = 2,500), beyond by the sort above.
 
 constexpr int kXyMax = 8192;
 constexpr int kXyThreads = 256;
@@ -870,10 +1180,22 @@ __global__ void order_xy_scatter_kernel(const int* __restrict__ rank, int D, int
     if (i < D) perm[rank[i]] = i;
 }
 
-size_t order_xy_scratch_bytes(int64_t D) { return sizeof(int) * (size_t)(D > 0 ? D : 1); }
+struct XyKeys {
+    const double* sites;
+    __device__ void load(int s, unsigned long long& a, unsigned long long& b, int& i) const {
+        a = ord_key(sites[2 * (int64_t)s]);
+        b = ord_key(sites[2 * (int64_t)s + 1]);
+        i = s;
+    }
+};
+
+size_t order_xy_scratch_bytes(int64_t D) {
+    return D > kXyMax ? sort_scratch_bytes(D, true) : sizeof(int) * (size_t)(D > 0 ? D : 1);
+}
 
 cudaError_t launch_order_xy(const double* sites, int64_t D, int32_t* perm, void* scratch, cudaStream_t st) {
-    if (D <= 0 || D > kXyMax) return cudaErrorInvalidValue;
+    if (D <= 0 || D > INT_MAX / 2) return cudaErrorInvalidValue;
+    if (D > kXyMax) return launch_sort<true>(XyKeys{sites}, D, perm, scratch, st);
     int* rank = (int*)scratch;
     cudaError_t e = cudaMemsetAsync(rank, 0, sizeof(int) * (size_t)D, st);
     if (e != cudaSuccess) return e;
