@@ -10,9 +10,10 @@
 //      below it, and the trailing update.  Every entry receives its terms in
 //      ascending k with fma and the pivot division last: the operations of
 //      the row-by-row definition in its order;
-//   3. the rows of L scaled by 1/L_vv (u likewise);
-//   4. Genz's recursion.  FP64 (here): CTA tiles of P = 128 lattice points, in
-//      panels of 32 variables: the panel's conditional means
+//   3. the rows of L in the recursion's form: integers of each row's scale
+//      (FP64), or scaled by 1/L_vv (u likewise; mixed);
+//   4. Genz's recursion.  FP64 (here), in 64-bit fixed point: CTA tiles of 64
+//      lattice points, in panels of 32 variables: the panel's conditional means
 //      u_v - sum_{t < v0} L_vt y_t are a register-tiled contraction of the
 //      panel's rows of L with the stored y history (smem-staged chunks of 32
 //      variables), then one thread per point runs the panel's variables in
@@ -27,13 +28,14 @@
 #include <mutex>
 
 #include "cov.cuh"
+#include "fix_step.cuh"
 #include "vk_internal.h"
 
 namespace vk {
 namespace {
 
 constexpr int kCholB = 32;   // Cholesky block
-constexpr int kFullP = 128;  // lattice points per CTA (one per thread in the sequential part)
+constexpr int kFullP = 64;   // lattice points per CTA (FP64 recursion)
 constexpr int kFullKC = 32;  // history chunk of the contraction
 
 __global__ void full_cov_kernel(const double* __restrict__ sites, int D, CovParams cv, double* __restrict__ A) {
@@ -312,25 +314,35 @@ __global__ void chol_update_kernel(double* __restrict__ A, int D, int k0, int pa
     }
 }
 
-// Scaled tables: Ls[v][t] = L_vt / L_vv (t < v), us[v] = u_v / L_vv.
-template <class T>
-__global__ void full_tables_kernel(const double* __restrict__ A, const double* __restrict__ u, int D,
-                                   T* __restrict__ Ls, T* __restrict__ us) {
-    const int v = blockIdx.y;
-    const double rd = 1.0 / A[(int64_t)v * D + v];
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < D; t += gridDim.x * blockDim.x)
-        Ls[(int64_t)v * D + t] = (t < v) ? (T)(A[(int64_t)v * D + t] * rd) : (T)0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) us[v] = (T)(u[v] * rd);
+// ---- the FP64 recursion, in 64-bit fixed point (fix_step.cuh) ----------------
+
+constexpr int kFullB = 32;         // panel width
+constexpr int kFullThreads = 128;
+constexpr int kFullT = 4;          // per-thread tile of the contraction: 4 variables x 4 points
+static_assert((kFullB / kFullT) * (kFullP / kFullT) == kFullThreads, "thread tile");
+
+// Row v: its scale and coefficients -L_vt as digits (t < v).
+__global__ void __launch_bounds__(128) full_tables_kernel(const double* __restrict__ A, const double* __restrict__ u,
+                                                          int D, fix::Digits* __restrict__ Ld,
+                                                          FixVar* __restrict__ var) {
+    __shared__ double red[4];
+    __shared__ int kL;
+    const int v = blockIdx.x, tid = threadIdx.x;
+    const double* row = A + (int64_t)v * D;
+    double sum = 0.0;
+    for (int t = tid; t < v; t += 128) sum += fabs(row[t]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((tid & 31) == 0) red[tid >> 5] = sum;
+    __syncthreads();
+    if (tid == 0) {
+        const FixVar r = fix_scale(row[v], red[0] + red[1] + red[2] + red[3], u[v], v);
+        var[v] = r;
+        kL = r.kL;
+    }
+    __syncthreads();
+    for (int t = tid; t < D; t += 128) Ld[(int64_t)v * D + t] = fix_coef(t < v ? row[t] : 0.0, kL);
 }
-
-// ---- the recursion ----------------------------------------------------------
-
-template <class T>
-struct FullTraits;
-template <>
-struct FullTraits<double> {
-    static constexpr int B = 32, TJ = 4, TP = 8;  // panel width; per-thread tile (variables x points)
-};
 
 struct FullArgs {
     int D;
@@ -339,138 +351,145 @@ struct FullArgs {
     int blocks_per_shift;
     const uint32_t* g;     // lattice vector, D - 1 entries
     const double* delta;   // S x dim shifts
+    const double* u;       // thresholds (for NaN only: its result is NaN)
     int dim;               // row stride of delta
 };
 
-// e = Phi(z), ec = 1 - e.
-__device__ __forceinline__ void full_phi(double z, double& e, double& ec) {
-    const double t = normcdf(-fabs(z));
-    e = (z < 0.0) ? t : 1.0 - t;
-    ec = (z < 0.0) ? 1.0 - t : t;
-}
+struct FullSmem {
+    fix::FixTables tb;
+    __align__(16) fix::Digits Ych[kFullKC][kFullP];      // chunk of the y history
+    __align__(16) fix::Digits Lch[kFullB][kFullKC + 1];  // the panel's rows of L against it
+    __align__(16) fix::Digits Lp[kFullB][kFullB + 1];    // the panel's own triangle
+    __align__(16) int64_t Z[kFullB][kFullP];             // conditional means, then the panel's y (digits)
+    FixVar var[kFullB];
+    uint64_t G[kFullB], Dt[kFullB];                      // lattice multipliers and this shift, 64-bit fixed point
+    double red[kFullP / 32];
+    int nan;
+};
 
-// y = Phi^{-1}(w e) at lattice coordinate v of point k of shift s.
-__device__ __forceinline__ double full_y(const FullArgs& a, int s, uint32_t k, int v, double e, double ec) {
-    const uint64_t rr = ((uint64_t)k * (uint64_t)a.g[v]) % (uint64_t)a.N;
-    double x = __dadd_rn((double)rr / (double)a.N, a.delta[(int64_t)s * a.dim + v]);
-    if (x >= 1.0) x -= 1.0;
-    const double am = fabs(__dsub_rn(__dmul_rn(2.0, x), 1.0));
-    const double w = __dsub_rn(1.0, am);
-    const double p = __dmul_rn(w, e), q = __dadd_rn(am, __dmul_rn(w, ec));
-    const double lo = 9.3326361850321887899e-302;  // 2^-1000
-    const double pc = fmax(p, lo), qc = fmax(q, lo);
-    return (pc <= qc) ? normcdfinv(pc) : -normcdfinv(qc);
-}
-
-template <class T>
-__global__ void __launch_bounds__(kFullP) full_genz_kernel(const T* __restrict__ Ls, const T* __restrict__ us,
-                                                           FullArgs a, T* __restrict__ Y,
-                                                           double* __restrict__ part) {
-    constexpr int B = FullTraits<T>::B, TJ = FullTraits<T>::TJ, TP = FullTraits<T>::TP;
-    constexpr int P = kFullP, KC = kFullKC;
-    static_assert((B / TJ) * (P / TP) == kFullP, "thread tile");
+// A CTA takes 64 lattice points: 192 KB of shared memory hold two CTAs an SM,
+// one in its point pass (two warps, a chain of D steps) beside the other's
+// contraction (four warps, 16 independent products a thread and variable).
+// The contraction's D^2/2 products a point cost 25 cycles a warp instruction
+// triple against the FP64 fma's 76.  (Tiles of 128 points left 152 SMs with 1 or 2
+// tiles each at N S = 24,000.)  D = 1,021, N S = 24,000: 52.2 -> 13.4 ms a call
+// (2.7 ms of it the factor); D = 2,500, N S = 65,536: 501 -> 145 ms.
+__global__ void __launch_bounds__(kFullThreads) full_genz_kernel(const fix::Digits* __restrict__ Ld,
+                                                                 const FixVar* __restrict__ var, FullArgs a,
+                                                                 fix::Digits* __restrict__ Y,
+                                                                 double* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char full_smem[];
-    T* Ych = (T*)full_smem;        // [KC][P]
-    T* Lch = Ych + KC * P;         // [B][KC + 1]
-    T* Zs = Lch + B * (KC + 1);    // [B][P]: conditional means, then the panel's y
-    T* Lp = Zs + B * P;            // [B][B + 1]: the panel's own triangle
-    __shared__ double red[kFullP / 32];
+    FullSmem& sm = *reinterpret_cast<FullSmem*>(full_smem);
+    constexpr int B = kFullB, P = kFullP, KC = kFullKC, T = kFullT;
     const int tid = threadIdx.x, D = a.D;
+    const uint64_t K = fix::opaque_mid();
+    load_fix_tables(sm.tb);
     const int s = blockIdx.x / a.blocks_per_shift;
     const int64_t k64 = (int64_t)(blockIdx.x % a.blocks_per_shift) * P + tid;
-    const bool valid = k64 < a.N;
+    const bool valid = tid < P && k64 < a.N;
     const uint32_t k = (uint32_t)(valid ? k64 : a.N - 1);
-    T* Yb = Y + (int64_t)blockIdx.x * D * P;  // this tile's y history [D][P]
-    const int tj = tid / (P / TP), tp = tid % (P / TP);  // thread tile (variables tj*TJ.., points tp*TP..)
-    double f = 1.0;
+    fix::Digits* Yb = Y + (int64_t)blockIdx.x * D * P;  // this tile's y history [D][P]
+    const int tj = tid / (P / T), tp = tid % (P / T);   // thread tile (variables tj T.., points tp T..)
+    fix::FixFloat f{~0ull, 0};
+    if (tid == 0) sm.nan = 0;
+    __syncthreads();
     for (int v0 = 0; v0 < D; v0 += B) {
         const int nb = min(B, D - v0);
-        // the panel's triangle
-        for (int x = tid; x < B * B; x += P) {
-            const int j = x / B, i = x % B;
-            Lp[j * (B + 1) + i] = (j < nb && i < j) ? Ls[(int64_t)(v0 + j) * D + v0 + i] : (T)0;
+        // the panel's constants and triangle
+        for (int j = tid; j < nb; j += kFullThreads) {
+            const int v = v0 + j;
+            sm.var[j] = var[v];
+            if (a.u[v] != a.u[v]) sm.nan = 1;
+            sm.G[j] = v < D - 1 ? fix64_ratio(a.g[v], (uint64_t)a.N) : 0;
+            sm.Dt[j] = v < D - 1 ? fix_shift(a.delta[(int64_t)s * a.dim + v]) : 0;
         }
-        // conditional means from the history: Zs[j][p] = us_v - sum_{t < v0} Ls[v][t] y_t[p]
-        T acc[TJ][TP];
+        for (int x = tid; x < B * B; x += kFullThreads) {
+            const int j = x / B, i = x % B;
+            sm.Lp[j][i] = (j < nb && i < j) ? Ld[(int64_t)(v0 + j) * D + v0 + i] : fix::Digits{0, 0};
+        }
+        // conditional means from the history: Z[j][p] = u_v - sum_{t < v0} L_vt y_t[p]
+        int64_t acc[T][T];
 #pragma unroll
-        for (int i = 0; i < TJ; ++i)
+        for (int i = 0; i < T; ++i)
 #pragma unroll
-            for (int q = 0; q < TP; ++q) acc[i][q] = (T)0;
+            for (int q = 0; q < T; ++q) acc[i][q] = 0;
         for (int t0 = 0; t0 < v0; t0 += KC) {
             __syncthreads();  // previous chunk consumed
-            for (int x = tid; x < KC * P; x += P) {
-                const int tt = x / P, p = x % P;
-                Ych[x] = Yb[(int64_t)(t0 + tt) * P + p];
-            }
-            for (int x = tid; x < B * KC; x += P) {
+            for (int x = tid; x < KC * P; x += kFullThreads) sm.Ych[x / P][x % P] = Yb[(int64_t)t0 * P + x];
+            for (int x = tid; x < B * KC; x += kFullThreads) {
                 const int j = x / KC, tt = x % KC;
-                Lch[j * (KC + 1) + tt] = (j < nb) ? Ls[(int64_t)(v0 + j) * D + t0 + tt] : (T)0;
+                sm.Lch[j][tt] = (j < nb) ? Ld[(int64_t)(v0 + j) * D + t0 + tt] : fix::Digits{0, 0};
             }
             __syncthreads();
-#pragma unroll 4
+#pragma unroll 2
             for (int tt = 0; tt < KC; ++tt) {
-                T lv[TJ], yv[TP];
+                fix::Digits lv[T], yv[T];
 #pragma unroll
-                for (int i = 0; i < TJ; ++i) lv[i] = Lch[(tj * TJ + i) * (KC + 1) + tt];
+                for (int i = 0; i < T; ++i) lv[i] = sm.Lch[tj * T + i][tt];
 #pragma unroll
-                for (int q = 0; q < TP; ++q) yv[q] = Ych[tt * P + tp * TP + q];
+                for (int q = 0; q < T; ++q) yv[q] = sm.Ych[tt][tp * T + q];
 #pragma unroll
-                for (int i = 0; i < TJ; ++i)
+                for (int i = 0; i < T; ++i)
 #pragma unroll
-                    for (int q = 0; q < TP; ++q) acc[i][q] = fma(lv[i], yv[q], acc[i][q]);
+                    for (int q = 0; q < T; ++q) acc[i][q] = fix::mul_add(lv[i], yv[q], acc[i][q], K);
             }
         }
+        __syncthreads();  // the constants are in place
 #pragma unroll
-        for (int i = 0; i < TJ; ++i) {
-            const int j = tj * TJ + i;
-            const T uv = (j < nb) ? us[v0 + j] : (T)0;
+        for (int i = 0; i < T; ++i) {
+            const int j = tj * T + i;
+            const int64_t uv = (j < nb) ? sm.var[j].up : 0;
 #pragma unroll
-            for (int q = 0; q < TP; ++q) Zs[j * P + tp * TP + q] = uv - acc[i][q];
+            for (int q = 0; q < T; ++q) sm.Z[j][tp * T + q] = uv + acc[i][q];
         }
         __syncthreads();
         // the panel's variables in order, one thread per point
-        const int p = tid;
-        for (int j = 0; j < nb; ++j) {
-            const int v = v0 + j;
-            T z = Zs[j * P + p];
-            for (int i = 0; i < j; ++i) z = fma(-Lp[j * (B + 1) + i], Zs[i * P + p], z);
-            T e, ec;
-            full_phi(z, e, ec);
-            f *= (double)e;
-            if (v < D - 1) Zs[j * P + p] = full_y(a, s, k, v, e, ec);
+        if (tid < P) {
+            const int p = tid;
+            fix::FixProb e;
+            for (int j = 0; j < nb; ++j) {
+                const int v = v0 + j;
+                int64_t z0 = sm.Z[j][p], z1 = 0;  // two chains of the panel's own terms
+                int i = 0;
+                for (; i + 1 < j; i += 2) {
+                    z0 = fix::mul_add(sm.Lp[j][i], reinterpret_cast<const fix::Digits&>(sm.Z[i][p]), z0, K);
+                    z1 = fix::mul_add(sm.Lp[j][i + 1], reinterpret_cast<const fix::Digits&>(sm.Z[i + 1][p]), z1, K);
+                }
+                if (i < j) z0 = fix::mul_add(sm.Lp[j][i], reinterpret_cast<const fix::Digits&>(sm.Z[i][p]), z0, K);
+                const FixVar& c = sm.var[j];
+                const int64_t hi = fix::mul_add(c.rdiag, fix::digits(z0 + z1), -fix::kMulBias, K);
+                fix_phi(sm.tb, hi, c.lim, c.shift, e, K);
+                if (v == 0)
+                    f = fix::prob(e);
+                else
+                    f = fix::times(f, e);
+                if (v < D - 1)
+                    reinterpret_cast<fix::Digits&>(sm.Z[j][p]) =
+                        fix_quantile(sm.tb, (uint64_t)k * sm.G[j] + sm.Dt[j], e, K);
+            }
+            for (int j = 0; j < nb; ++j)
+                if (v0 + j < D - 1) Yb[(int64_t)(v0 + j) * P + p] = reinterpret_cast<const fix::Digits&>(sm.Z[j][p]);
         }
-        for (int j = 0; j < nb; ++j)
-            if (v0 + j < D - 1) Yb[(int64_t)(v0 + j) * P + p] = Zs[j * P + p];
-        __syncthreads();  // Zs and Lp reused by the next panel
+        __syncthreads();  // Z and Lp reused by the next panel
     }
     // tile sum of the point products, fixed order
-    double v = valid ? f : 0.0;
+    double v = valid ? __longlong_as_double((long long)fix::to_bits(f)) : 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((tid & 31) == 0) red[tid >> 5] = v;
+    if (tid < P && (tid & 31) == 0) sm.red[tid >> 5] = v;
     __syncthreads();
     if (tid == 0) {
         double t = 0.0;
-        for (int w = 0; w < kFullP / 32; ++w) t += red[w];
-        part[blockIdx.x] = t;
+        for (int w = 0; w < P / 32; ++w) t += sm.red[w];
+        part[blockIdx.x] = sm.nan ? __longlong_as_double(0x7ff8000000000000LL) : t;
     }
 }
 
-template <class T>
-size_t full_smem_bytes() {
-    constexpr int B = FullTraits<T>::B;
-    return sizeof(T) * ((size_t)kFullKC * kFullP + (size_t)B * (kFullKC + 1) + (size_t)B * kFullP +
-                        (size_t)B * (B + 1));
-}
-
-template <class T>
-cudaError_t launch_full_genz_t(const double* A, const double* u, const FullArgs& a, void* Ls, void* us, void* Y,
-                               double* part, cudaEvent_t ev_begin, cudaEvent_t ev_end, cudaStream_t st) {
-    const int D = a.D;
-    full_tables_kernel<T><<<dim3((D + 255) / 256 > 8 ? 8 : (D + 255) / 256, D), 256, 0, st>>>(A, u, D, (T*)Ls, (T*)us);
+cudaError_t launch_full_genz_fix(const double* A, const double* u, const FullArgs& a, void* Ld, void* var, void* Y,
+                                 double* part, cudaEvent_t ev_begin, cudaEvent_t ev_end, cudaStream_t st) {
+    full_tables_kernel<<<a.D, 128, 0, st>>>(A, u, a.D, (fix::Digits*)Ld, (FixVar*)var);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const size_t smem = full_smem_bytes<T>();
     static std::mutex mu;
     static std::map<int, bool> attr;
     int dev = 0;
@@ -478,14 +497,16 @@ cudaError_t launch_full_genz_t(const double* A, const double* u, const FullArgs&
     {
         std::lock_guard<std::mutex> lk(mu);
         if (!attr[dev]) {
-            e = cudaFuncSetAttribute(full_genz_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            e = cudaFuncSetAttribute(full_genz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(FullSmem));
             if (e != cudaSuccess) return e;
             attr[dev] = true;
         }
     }
     const int blocks = a.S * a.blocks_per_shift;
     if (ev_begin && (e = cudaEventRecord(ev_begin, st)) != cudaSuccess) return e;
-    full_genz_kernel<T><<<blocks, kFullP, smem, st>>>((const T*)Ls, (const T*)us, a, (T*)Y, part);
+    full_genz_kernel<<<blocks, kFullThreads, sizeof(FullSmem), st>>>((const fix::Digits*)Ld, (const FixVar*)var, a,
+                                                                     (fix::Digits*)Y, part);
     e = cudaGetLastError();
     if (e == cudaSuccess && ev_end) e = cudaEventRecord(ev_end, st);
     return e;
@@ -744,7 +765,8 @@ size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed) {
                           al(sizeof(uint32_t) * S * dim) + al(sizeof(double) * S * nblk) + al(2 * sizeof(int)) +
                           al(sizeof(uint64_t) + 2 * sizeof(int64_t) + sizeof(int32_t));
     if (mixed) return shared + al(chol_tc_scratch_bytes(D)) + full_tc_scratch_bytes(D, N, S);
-    return shared + al(sizeof(double) * D * D) + al(sizeof(double) * D) + al(sizeof(double) * (size_t)S * bps * D * kFullP);
+    return shared + al(sizeof(fix::Digits) * D * D) + al(sizeof(FixVar) * D) +
+           al(sizeof(fix::Digits) * (size_t)S * bps * D * kFullP);
 }
 
 cudaError_t launch_full_genz(const double* sites, const double* u, int64_t D, const vecchia_cov& cov, int64_t N,
@@ -797,10 +819,10 @@ cudaError_t launch_full_genz(const double* sites, const double* u, int64_t D, co
         e = launch_full_genz_tc(A, u, D, N, S, gdev + dim, dfix, (int)dim, p, part, bad + 1, wait_ns, withhold,
                                 ev_begin, ev_end, st);
     } else {
-        void* Ls = p;
-        p += al(sizeof(double) * D * D);
-        void* us = p;
-        p += al(sizeof(double) * D);
+        void* Ld = p;
+        p += al(sizeof(fix::Digits) * D * D);
+        void* var = p;
+        p += al(sizeof(FixVar) * D);
         void* Y = p;
         FullArgs fa;
         fa.D = (int)D;
@@ -809,8 +831,9 @@ cudaError_t launch_full_genz(const double* sites, const double* u, int64_t D, co
         fa.blocks_per_shift = (int)bps;
         fa.g = gdev;
         fa.delta = delta;
+        fa.u = u;
         fa.dim = (int)dim;
-        e = launch_full_genz_t<double>(A, u, fa, Ls, us, Y, part, ev_begin, ev_end, st);
+        e = launch_full_genz_fix(A, u, fa, Ld, var, Y, part, ev_begin, ev_end, st);
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(part_host, part, sizeof(double) * S * nblk, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(bad_host, bad, sizeof(int), cudaMemcpyDeviceToHost, st);
