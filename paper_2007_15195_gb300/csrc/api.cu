@@ -302,39 +302,6 @@ uint32_t* lattice_for(vecchia_ctx* c, int64_t N) {
     return d;
 }
 
-// Built-in tile (measured on the 50x50 grid): mixed blocks of up to 32
-// variables run two points per lane (one vote per step for both), 4 warps up
-// to 21 variables and 8 above; FP64 one point, up to 8 warps with the shifts
-// spread evenly (its function tables take 45 KB a CTA, so 16 resident warps want
-// two CTAs of 8: 55.6 against 58.2 ms with 4 warps at m = 20).  Shift groups (a power
-// of two, so S = 2^k splits evenly) until a launch has ~2048 CTA items, never
-// fewer shifts per item than warps (a warp without a unit idles); ~4096 items
-// for blocks of up to 16 variables, which fit more CTAs per SM.  Blocks
-// above 32 variables: 8 warps, one point per lane, every shift of a term in
-// one item, so the one-warp Cholesky of up to 64 variables is shared by the
-// most work.
-GenzTile default_tile(bool mixed, int64_t total_sites, int max_S, int bucket) {
-    GenzTile t;
-    const int dmax = vk::kDmaxBuckets[bucket];
-    if (dmax > 32) {
-        t.warps = 8;
-        t.points = 1;
-        t.slices = 1;
-        t.groups = 1;
-        return t;
-    }
-    const int rounds = (max_S + 7) / 8;
-    t.warps = mixed ? (dmax > 21 ? 8 : 4) : (max_S + rounds - 1) / rounds;
-    t.points = mixed ? 2 : 1;
-    t.slices = 1;
-    // small blocks fit more CTAs per SM: they want more items
-    const int64_t target = dmax <= 16 ? 4096 : 2048;
-    int g = 1;
-    while (g < max_S && (int64_t)g * total_sites < target && max_S / (2 * g) >= t.warps) g *= 2;
-    t.groups = g;
-    return t;
-}
-
 // ------------------------------ the pipeline --------------------------------
 // A batch of n problems: validation and buckets (Batch, prepare), a layout of
 // one device arena and one host parameter blob, and the launch sequence
@@ -416,7 +383,8 @@ int prepare(vecchia_ctx* c, const vecchia_problem* probs, int n, int precision, 
     int max_groups = 1;
     for (int b = 0; b < NB; ++b) {
         B.tiles[b] = c->tile_set[B.mixed][b] ? c->tile[B.mixed][b]
-                                             : default_tile(B.mixed, B.total_sites, std::max(B.max_S[b], 2), b);
+                                             : vk::default_tile(B.mixed, B.total_sites, std::max(B.max_S[b], 2), b,
+                                                            vk::device_sm_count(c ? c->device : 0));
         max_groups = std::max(max_groups, B.tiles[b].groups);
     }
     B.fb_cap = B.mixed ? B.total_sites * max_groups + vk::genz_items_slack(vk::device_sm_count(c ? c->device : 0)) : 0;
@@ -1134,7 +1102,11 @@ int vecchia_log_cdf_unordered(vecchia_ctx* c, const double* sites, const double*
     }
     // ordering, queued on the stream
     std::vector<int32_t> hp;
-    if (e == cudaSuccess) {
+    const bool small = order_kind == VECCHIA_ORDER_XY && D <= vk::kSmallMax;
+    if (e == cudaSuccess && small) {
+        e = vk::launch_order_small(sd, ud, D, perm, so, uo, X + o_scr, s);
+        if (e == cudaSuccess && m > 0) e = vk::launch_knn_small(D, m, nbr, X + o_scr, s);
+    } else if (e == cudaSuccess) {
         if (order_kind == VECCHIA_ORDER_MAXMIN) {
             e = vk::launch_maxmin(sd, D, perm, X + o_scr, s);
         } else if (order_kind == VECCHIA_ORDER_XY) {
@@ -1145,9 +1117,11 @@ int vecchia_log_cdf_unordered(vecchia_ctx* c, const double* sites, const double*
             e = cudaMemcpyAsync(perm, hp.data(), sizeof(int32_t) * D, cudaMemcpyHostToDevice, s);
         }
     }
-    if (e == cudaSuccess) e = cudaMemsetAsync(X + o_bad, 0, sizeof(int), s);
-    if (e == cudaSuccess) e = vk::launch_gather(perm, sd, ud, D, so, uo, (int*)(X + o_bad), s);
-    if (e == cudaSuccess && m > 0) e = vk::launch_knn(so, D, m, nbr, X + o_scr, s);
+    if (!small) {
+        if (e == cudaSuccess) e = cudaMemsetAsync(X + o_bad, 0, sizeof(int), s);
+        if (e == cudaSuccess) e = vk::launch_gather(perm, sd, ud, D, so, uo, (int*)(X + o_bad), s);
+        if (e == cudaSuccess && m > 0) e = vk::launch_knn(so, D, m, nbr, X + o_scr, s);
+    }
     if (e == cudaSuccess && !hp.empty()) e = cudaStreamSynchronize(s);  // hp must outlive its upload
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1743,7 +1717,8 @@ int vecchia_partials_async(vecchia_ctx* c, const vecchia_segment* segs, int n, i
     int max_groups = 1;
     for (int b = 0; b < NB; ++b) {
         tiles[b] = c->tile_set[mixed][b] ? c->tile[mixed][b]
-                                         : default_tile(mixed, total_sites, std::max(max_S[b], 2), b);
+                                         : vk::default_tile(mixed, total_sites, std::max(max_S[b], 2), b,
+                                                        vk::device_sm_count(c->device));
         max_groups = std::max(max_groups, tiles[b].groups);
     }
     const int64_t fb_cap =

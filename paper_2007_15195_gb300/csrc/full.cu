@@ -28,6 +28,7 @@
 #include <mutex>
 
 #include "cov.cuh"
+#include "exact_math.h"
 #include "fix_step.cuh"
 #include "vk_internal.h"
 
@@ -55,21 +56,6 @@ __device__ __forceinline__ void tri_rc(int e, int& r, int& c) {
     c = e - r * (r + 1) / 2;
 }
 
-// 1/sqrt(s) for a positive normal double: the hardware approximation
-// (rsqrt.approx.f64, about 2^-22 relative) and two Newton-Raphson steps
-// y <- y + y (1 - s y^2) / 2, each squaring the relative error -- inline (a
-// library call would spill the caller's registers around it).
-__device__ __forceinline__ double rsqrt_nr(double s) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const double r = fma(-(s * y), y, 1.0);
-        y = fma(0.5 * y, r, y);
-    }
-    return y;
-}
-
 // The pairs (row, column) of a packed lower triangle, in packed order: the
 // pairs of an n x n triangle are the table's first n (n + 1) / 2 entries.
 __device__ __forceinline__ void pair_table(unsigned short* tab) {
@@ -81,47 +67,49 @@ __device__ __forceinline__ void pair_table(unsigned short* tab) {
 }
 
 // Factor the b x b block T in shared memory, all threads of the CTA,
-// right-looking: at step j the column below the pivot is divided by it (FAST:
-// multiplied by its reciprocal square root, a shorter dependent chain on
-// GB300's 1/64-rate FP64 unit than a square root and a division), then the
-// packed trailing triangle takes one fma per entry, spread over the threads
-// through the pair table.  (Taking the next pivot's root inside the trailing
-// update, by the thread that updates that entry, was slower: 31 against 26 us
-// a block.)  Returns the first non-positive pivot, or -1.
-template <bool FAST>
+// right-looking: at step j the column below the pivot is divided by it
+// (exact_math.h: the same values as the FP64 square root and division by a
+// shorter chain of integer instructions), then the packed trailing triangle
+// takes one fma per entry, spread over the threads through the pair table.
+// Warp 0 updates the next column first and goes on to its pivot while the other
+// warps take the rest, so a step costs warp 0's chain and one barrier.  Returns
+// the first non-positive pivot, or -1.
 __device__ int factor_block(double (*T)[kCholB + 1], const unsigned short* tab, int b) {
     const int tid = threadIdx.x;
     for (int j = 0; j < b; ++j) {
-        const double s = T[j][j];
-        if (!(s > 0.0)) return j;  // block-uniform
-        double piv = 0.0;
-        if (tid < 32) {  // the pivot and its column: one warp (the others would only repeat it)
-            if constexpr (FAST) {
-                const double rs = rsqrt_nr(s);
-                piv = s * rs;
-                if (tid < b - 1 - j) T[j + 1 + tid][j] = T[j + 1 + tid][j] * rs;
+        int failed = 0;
+        if (tid < 32) {
+            const double s = T[j][j];
+            if (s > 0.0) {
+                const exact::Pivot piv = exact::pivot(s);
+                if (tid < b - 1 - j) T[j + 1 + tid][j] = exact::quotient(T[j + 1 + tid][j], piv);
+                __syncwarp();
+                if (tid == 0) T[j][j] = piv.piv;
             } else {
-                piv = sqrt(s);
-                if (tid < b - 1 - j) T[j + 1 + tid][j] = T[j + 1 + tid][j] / piv;
+                failed = 1;
             }
         }
-        __syncthreads();
-        if (tid == 0) T[j][j] = piv;
-        const int n = b - 1 - j;
-        for (int e = tid; e < n * (n + 1) / 2; e += blockDim.x) {
-            const unsigned t = tab[e];
-            const int r = j + 1 + (int)(t >> 8), cc = j + 1 + (int)(t & 255u);
-            T[r][cc] = fma(-T[r][j], T[cc][j], T[r][cc]);
+        if (__syncthreads_or(failed)) return j;  // block-uniform
+        if (tid < 32) {
+            if (tid < b - 1 - j) T[j + 1 + tid][j + 1] = fma(-T[j + 1 + tid][j], T[j + 1][j], T[j + 1 + tid][j + 1]);
+            __syncwarp();
+        } else {
+            const int n = b - 2 - j;
+            for (int e = tid - 32; e < n * (n + 1) / 2; e += blockDim.x - 32) {
+                const unsigned t = tab[e];
+                const int r = j + 2 + (int)(t >> 8), cc = j + 2 + (int)(t & 255u);
+                T[r][cc] = fma(-T[r][j], T[cc][j], T[r][cc]);
+            }
         }
-        __syncthreads();
     }
+    __syncthreads();
     return -1;
 }
 
 // The diagonal block at k0, 512 threads (one trailing entry a thread at the
 // first pivots, so thread 0 holds only the next pivot).  FP64 path: each entry of the factor
-// receives its terms in ascending order with fma and the pivot division last;
-// FAST (mixed path): pivots from reciprocal square roots.  (Tried for the
+// receives its terms in ascending order with fma and the pivot division last.
+// (Tried for the
 // mixed path and slower: one warp holding the block in registers and
 // shuffling the columns, 49 against 26 us a block, all its FP64 work on one
 // SMSP; the factor repeated by every CTA of the row solve, 70 us a block
@@ -131,7 +119,6 @@ __device__ int factor_block(double (*T)[kCholB + 1], const unsigned short* tab, 
 // column order), which the tensor-core update of that column leaves out, so
 // that this factor waits only for the row solve of the column before and not
 // for the update of its whole first tile column.
-template <bool FAST>
 __global__ void __launch_bounds__(512) chol_diag_kernel(double* __restrict__ A, int D, int k0,
                                                         int* __restrict__ bad, int upd) {
     __shared__ double T[kCholB][kCholB + 1];
@@ -161,7 +148,7 @@ __global__ void __launch_bounds__(512) chol_diag_kernel(double* __restrict__ A, 
         }
         __syncthreads();
     }
-    const int fail = factor_block<FAST>(T, tab, b);
+    const int fail = factor_block(T, tab, b);
     if (fail >= 0) {
         if (threadIdx.x == 0) atomicMin(bad, k0 + fail);
         return;
@@ -182,6 +169,7 @@ __global__ void __launch_bounds__(512) chol_diag_kernel(double* __restrict__ A, 
 // last bits, and with them which exactly singular block is reported).
 __global__ void chol_trsm_kernel(double* __restrict__ A, int D, int k0) {
     __shared__ double Lk[kCholB][kCholB + 1];
+    __shared__ exact::Pivot piv[kCholB];
     // the diagonal block, a row per thread and pass with its 32 loads issued
     // together (a CTA has as few as 8 threads: a load loop would wait on L2
     // 128 times in sequence)
@@ -192,6 +180,7 @@ __global__ void chol_trsm_kernel(double* __restrict__ A, int D, int k0) {
         for (int c = 0; c < kCholB; ++c) v[c] = (c <= r) ? src[c] : 0.0;
 #pragma unroll
         for (int c = 0; c < kCholB; ++c) Lk[r][c] = v[c];
+        piv[r] = exact::pivot_of(Lk[r][r]);
     }
     __syncthreads();
     const int r = k0 + kCholB + blockIdx.x * blockDim.x + threadIdx.x;
@@ -202,7 +191,7 @@ __global__ void chol_trsm_kernel(double* __restrict__ A, int D, int k0) {
     for (int j = 0; j < kCholB; ++j) x[j] = row[j];
 #pragma unroll
     for (int j = 0; j < kCholB; ++j) {
-        x[j] = x[j] / Lk[j][j];
+        x[j] = exact::quotient(x[j], piv[j]);
 #pragma unroll
         for (int k = j + 1; k < kCholB; ++k) x[k] = fma(-x[j], Lk[k][j], x[k]);
     }
@@ -565,7 +554,7 @@ cudaError_t enqueue_chol(double* A, int64_t D, int* bad, cudaStream_t st, void* 
     const int64_t nblk = (D + kCholB - 1) / kCholB;
     if (nblk <= 2 || e != cudaSuccess) {  // nothing to overlap
         for (int64_t k0 = 0; k0 < D && e == cudaSuccess; k0 += kCholB) {
-            chol_diag_kernel<false><<<1, 512, 0, st>>>(A, (int)D, (int)k0, bad, 0);
+            chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, (int)k0, bad, 0);
             const int64_t rows = D - k0 - kCholB;
             if (rows > 0) {
                 const int rb = trsm_rows_per_cta(rows, sms);
@@ -601,7 +590,7 @@ cudaError_t enqueue_chol(double* A, int64_t D, int* bad, cudaStream_t st, void* 
         // k + 1 (which applies column k's update to its own block), then the
         // solve of column k + 1 once the tensor-core update of column k + 1's
         // other rows (side2) is in.  side: the rest of the trailing update.
-        chol_diag_kernel<true><<<1, 512, 0, st>>>(A, (int)D, 0, bad, 0);
+        chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, 0, bad, 0);
         for (int64_t k = 0; k < nblk && e == cudaSuccess; ++k) {
             const int64_t k0 = k * kCholB, rows = D - k0 - kCholB;
             if (rows <= 0) break;
@@ -626,7 +615,7 @@ cudaError_t enqueue_chol(double* A, int64_t D, int* bad, cudaStream_t st, void* 
             // block k + 1, which the rest of step k - 1 has updated
             if (k > 0 && e == cudaSuccess) e = cudaStreamWaitEvent(st, ev_rest[(k - 1) & 1], 0);
             if (e == cudaSuccess) {
-                chol_diag_kernel<true><<<1, 512, 0, st>>>(A, (int)D, (int)(k0 + kCholB), bad, 1);
+                chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, (int)(k0 + kCholB), bad, 1);
                 e = cudaGetLastError();
             }
             if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev_p0[k & 1], 0);
@@ -634,7 +623,7 @@ cudaError_t enqueue_chol(double* A, int64_t D, int* bad, cudaStream_t st, void* 
     }
     for (int64_t k = 0; !tc && k < nblk && e == cudaSuccess; ++k) {
         const int64_t k0 = k * kCholB, rows = D - k0 - kCholB;
-        chol_diag_kernel<false><<<1, 512, 0, st>>>(A, (int)D, (int)k0, bad, 0);
+        chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, (int)k0, bad, 0);
         if (rows <= 0) {
             e = cudaGetLastError();
             break;
@@ -757,6 +746,18 @@ int64_t full_genz_blocks_per_shift(int64_t N, bool mixed) {
 
 // Scratch: the shared part (factor, lattice and shift tables, block sums,
 // status words) followed by the precision's own tables and y history.
+// FP64 recursion: the tensor cores' contraction from kFixTcMin variables on (XXX),
+// unless its history (16 bytes a y value, twice the integer form's) would not fit
+// beside other work.
+#ifndef VK_FIXTC
+#define VK_FIXTC 128
+#endif
+constexpr int64_t kFixTcMin = VK_FIXTC;
+constexpr size_t kFixTcMaxBytes = 96ull << 30;
+bool fix_tc_pays(int64_t D, int64_t N, int S) {
+    return D >= kFixTcMin && full_fix_tc_scratch_bytes(D, N, S) <= kFixTcMaxBytes;
+}
+
 size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed) {
     const int64_t bps = (N + kFullP - 1) / kFullP, nblk = full_genz_blocks_per_shift(N, mixed);
     const int64_t dim = D > 1 ? D - 1 : 1;
@@ -765,6 +766,7 @@ size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed) {
                           al(sizeof(uint32_t) * S * dim) + al(sizeof(double) * S * nblk) + al(2 * sizeof(int)) +
                           al(sizeof(uint64_t) + 2 * sizeof(int64_t) + sizeof(int32_t));
     if (mixed) return shared + al(chol_tc_scratch_bytes(D)) + full_tc_scratch_bytes(D, N, S);
+    if (fix_tc_pays(D, N, S)) return shared + full_fix_tc_scratch_bytes(D, N, S);
     return shared + al(sizeof(fix::Digits) * D * D) + al(sizeof(FixVar) * D) +
            al(sizeof(fix::Digits) * (size_t)S * bps * D * kFullP);
 }
@@ -818,6 +820,11 @@ cudaError_t launch_full_genz(const double* sites, const double* u, int64_t D, co
     if (mixed) {
         e = launch_full_genz_tc(A, u, D, N, S, gdev + dim, dfix, (int)dim, p, part, bad + 1, wait_ns, withhold,
                                 ev_begin, ev_end, st);
+    } else if (fix_tc_pays(D, N, S)) {
+        e = cudaMemsetAsync(part, 0, sizeof(double) * S * nblk, st);
+        if (e == cudaSuccess)
+            e = launch_full_fix_tc(A, u, D, N, S, gdev, delta, (int)dim, p, part, (int)nblk, bad + 1, wait_ns, ev_begin,
+                                   ev_end, st);
     } else {
         void* Ld = p;
         p += al(sizeof(fix::Digits) * D * D);

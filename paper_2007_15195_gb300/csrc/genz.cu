@@ -33,6 +33,7 @@
 #include <tuple>
 
 #include "cov.cuh"
+#include "exact_math.h"
 #include "fix_step.cuh"
 #include "special_f32.h"
 #include "vk_internal.h"
@@ -650,9 +651,20 @@ __device__ __forceinline__ bool term_block(GenzSmem<DMAX, MIXED>& sm, const Prob
     return __all_sync(0xffffffffu, ok);
 }
 
+// Lattice slices of a shift where the tile names none, of the problem's own S and
+// N alone (so a problem's sums do not depend on the batch it runs in): one in the
+// mixed fast form, whose FP32 lane sums another split would round anew; FP64 as
+// many as make the units (shifts x slices) a multiple of four warps; four in the
+// log-space form, whose few flagged terms run one to a CTA.
+__host__ __device__ constexpr int auto_slices(int S, int64_t N, int mode) {
+    int g = mode == kModeFast ? 1 : (mode == kModeSafe || (S & 1)) ? 4 : (S & 2) ? 2 : 1;
+    while (g > 1 && (S * g > kMaxUnits || N < 256 * g)) g >>= 1;
+    return g;
+}
+
 template <int DMAX, int P, int MODE>
 __global__ void __launch_bounds__(max_threads(DMAX, P, MODE)) __maxnreg__(reg_cap(DMAX, P, MODE))
-    genz_kernel(const ProbDev* __restrict__ probs, ItemSrc src, int slices, int max_S,
+    genz_kernel(const ProbDev* __restrict__ probs, ItemSrc src, int tile_slices, int max_S,
                 ProbResult* __restrict__ results, int* __restrict__ fallback_count,
                 int2* __restrict__ fallback_items) {
     constexpr bool MIXED = MODE != kModeFP64;
@@ -675,8 +687,9 @@ __global__ void __launch_bounds__(max_threads(DMAX, P, MODE)) __maxnreg__(reg_ca
         const int64_t term = item.y;
         const int S = Pd.S;
         const int s_lo = (S * grp) / groups, s_hi = (S * (grp + 1)) / groups;
+        const int slices = tile_slices > 0 ? tile_slices : auto_slices(S, Pd.N, MODE);
 
-        // ---- prologue: block (warp 0), covariance (all warps), Cholesky (warp 0); FP64 ----
+        // ---- prologue: block (warp 0), covariance and Cholesky (all warps); FP64 ----
         if (warp == 0) {
             int c = 0, d = 1;
             int64_t i0 = 0;
@@ -717,41 +730,49 @@ __global__ void __launch_bounds__(max_threads(DMAX, P, MODE)) __maxnreg__(reg_ca
             }
         }
         __syncthreads();
-        if (warp == 0 && !sm.bad) {
+        if (!sm.bad) {
             const int d = sm.q + 1;
-            int bad = 0;
             // Cholesky, right-looking: after column j is final, the trailing
-            // triangle takes its update fma(-L_rj, L_cj, A_rc), entries packed
-            // over the lanes.  Each entry thus receives its terms in ascending
-            // k with fma and is divided by the pivot last: the operations of
-            // the row-by-row definition, in its order.
+            // triangle takes its update fma(-L_rj, L_cj, A_rc).  Each entry thus
+            // receives its terms in ascending k with fma and is divided by the
+            // pivot last: the operations of the row-by-row definition, in its
+            // order.  Warp 0 takes the next column's entries and goes on to its
+            // pivot and quotients (exact_math.h: the same values by integers, a
+            // third of the FP64 chain), the other warps the rest of the triangle
+            // meanwhile; one barrier a column.  (One warp for all of it: 26 us a
+            // term at d = 21, 160 us at d = 51.)
+            int failed = 0;
             for (int j = 0; j < d; ++j) {
-                const double s = sm.A[j][j];
-                if (!(s > 0.0)) {  // warp-uniform: every lane reads the same value
-                    bad = 1;
-                    break;
+                if (warp == 0) {
+                    const double s = sm.A[j][j];
+                    if (s > 0.0) {  // warp-uniform: every lane reads the same value
+                        const exact::Pivot piv = exact::pivot(s);
+                        for (int r = j + 1 + lane; r < d; r += 32) sm.A[r][j] = exact::quotient(sm.A[r][j], piv);
+                        __syncwarp();
+                        if (lane == 0) sm.A[j][j] = piv.piv;
+                    } else {
+                        failed = 1;
+                    }
                 }
-                const double piv = sqrt(s);
-                for (int r = j + 1 + lane; r < d; r += 32) sm.A[r][j] = sm.A[r][j] / piv;
-                __syncwarp();
-                if (lane == 0) sm.A[j][j] = piv;
-                const int n = d - 1 - j;
-                for (int e = lane; e < n * (n + 1) / 2; e += 32) {
-                    int a, b;
-                    tri_index(e, a, b);
-                    const int r = j + 1 + a, col = j + 1 + b;
-                    sm.A[r][col] = fma(-sm.A[r][j], sm.A[col][j], sm.A[r][col]);
+                failed = __syncthreads_or(failed);
+                if (failed) break;  // CTA-uniform
+                if (warp == 0) {
+                    for (int r = j + 1 + lane; r < d; r += 32)
+                        sm.A[r][j + 1] = fma(-sm.A[r][j], sm.A[j + 1][j], sm.A[r][j + 1]);
+                    __syncwarp();
                 }
-                __syncwarp();
+                if (warp > 0 || n_warps == 1) {
+                    const int n = d - 2 - j, w = n_warps > 1 ? 32 : 0;
+                    for (int e = (int)threadIdx.x - w; e < n * (n + 1) / 2; e += (int)blockDim.x - w) {
+                        int a, b;
+                        tri_index(e, a, b);
+                        const int r = j + 2 + a, col = j + 2 + b;
+                        sm.A[r][col] = fma(-sm.A[r][j], sm.A[col][j], sm.A[r][col]);
+                    }
+                    if (n_warps == 1) __syncwarp();
+                }
             }
-            if (lane == 0) {
-                sm.bad = bad;
-                if (!bad) {
-                    const double z0 = sm.bu[0] / sm.A[0][0];
-                    phi_pair64(z0, sm.e0, sm.ec0);
-                    sm.le2_0 = (sm.e0 < 0x1p-64) ? (float)log2(sm.e0) : 0.0f;
-                }
-            }
+            if (failed && threadIdx.x == 0) sm.bad = 1;
         }
         __syncthreads();
         const int q = sm.q, c = sm.c;
@@ -763,6 +784,13 @@ __global__ void __launch_bounds__(max_threads(DMAX, P, MODE)) __maxnreg__(reg_ca
             // kZs z that its Phi takes; FP64: integers of each row's scale)
             constexpr int LS = GenzSmem<DMAX, MIXED>::LS;
             const int d = q + 1;
+            if (threadIdx.x == blockDim.x - 1) {  // e_0, beside the tables
+                const double z0 = sm.bu[0] / sm.A[0][0];
+                phi_pair64(z0, sm.e0, sm.ec0);
+                sm.le2_0 = (sm.e0 < 0x1p-64) ? (float)log2(sm.e0) : 0.0f;
+                if constexpr (!MIXED)
+                    sm.p0 = fix::prob_of((uint64_t)__double_as_longlong(z0 < 0.0 ? sm.e0 : sm.ec0), z0 < 0.0);
+            }
             if constexpr (MIXED) {
                 for (int v = threadIdx.x; v < DMAX; v += blockDim.x)
                     sm.diag[v] = (v < d) ? special::kZsD / sm.A[v][v] : 0.0;
@@ -772,10 +800,6 @@ __global__ void __launch_bounds__(max_threads(DMAX, P, MODE)) __maxnreg__(reg_ca
                         fix_row<DMAX>(sm, v, Pd.g[v - 1], (uint64_t)Pd.N);
                     else
                         sm.up[v] = 0;
-                }
-                if (threadIdx.x == 0) {
-                    const double z0 = sm.bu[0] / sm.A[0][0];
-                    sm.p0 = fix::prob_of((uint64_t)__double_as_longlong(z0 < 0.0 ? sm.e0 : sm.ec0), z0 < 0.0);
                 }
             }
             __syncthreads();
@@ -893,10 +917,13 @@ __global__ void __launch_bounds__(max_threads(DMAX, P, MODE)) __maxnreg__(reg_ca
 //   final: one warp per problem adds the slices in order and forms
 //     log P = sum_i T_i and SE = sqrt(sum_s l_s^2 / (S (S-1))).
 
-// One warp a slice: the per-site work (two FP64 logarithms and the S
-// delta-method quotients) is FP64-bound on GB300, so a 2,500-site problem is
-// spread over 79 SMs rather than 10.
+// The per-site work (two FP64 logarithms and the S delta-method quotients) is
+// FP64-bound on GB300: 32 sites a CTA, so that a 2,500-site problem is spread over
+// 79 SMs, and eight warps a CTA, the means and logarithms on two of them and the
+// shifts' quotients over all (S = 10: 16.7 -> 7.9 us).
 constexpr int kSliceSites = kLogsumSlice;
+constexpr int kLogsumWarps = 8;
+static_assert(kSliceSites == 32, "a lane a site");
 
 __device__ __forceinline__ double warp_sum_xor(double v) {
 #pragma unroll
@@ -904,69 +931,81 @@ __device__ __forceinline__ double warp_sum_xor(double v) {
     return v;
 }
 
-__global__ void __launch_bounds__(kSliceSites) logsum_partial_kernel(
+__global__ void __launch_bounds__(32 * kLogsumWarps) logsum_partial_kernel(
     const ProbDev* __restrict__ probs, double* const* __restrict__ terms, double* __restrict__ scratch,
     const int64_t* __restrict__ scratch_off) {
-    __shared__ double red[kMaxS + 1][kSliceSites / 32];
+    __shared__ double mean[2][kSliceSites], lg[2][kSliceSites];
     const int pi = blockIdx.y, slice = blockIdx.x;
     const ProbDev& Pd = probs[pi];
     const int64_t D = Pd.n_terms;
     const int S = Pd.S;
     if ((int64_t)slice * kSliceSites >= D) return;  // CTA-uniform
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t i = (int64_t)slice * kSliceSites + tid;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = (int64_t)slice * kSliceSites + lane;
     const bool valid = i < D;
-    double T = 0.0, a = 1.0, b = 1.0;
-    if (valid) {
-        double sn = 0.0, sd = 0.0;
-        for (int s = 0; s < S; ++s) {
-            sn += Pd.num[i * S + s];
-            sd += Pd.den[i * S + s];
+    if (warp < 2) {
+        double m = 1.0;
+        if (valid) {
+            const double* v = (warp == 0 ? Pd.num : Pd.den) + i * S;
+            double sum = 0.0;
+            for (int s = 0; s < S; ++s) sum += v[s];
+            m = sum / (double)S;
         }
-        a = sn / (double)S;
-        b = sd / (double)S;
-        T = log(a) - log(b);
-        if (terms && terms[pi]) terms[pi][i] = T;
-    }
-    double v = warp_sum_xor(T);
-    if (lane == 0) red[0][warp] = v;
-    for (int s = 0; s < S; ++s) {  // quotients, not products by reciprocals: equal shifts give exactly 0
-        const double c = valid ? Pd.num[i * S + s] / a - Pd.den[i * S + s] / b : 0.0;
-        v = warp_sum_xor(c);
-        if (lane == 0) red[1 + s][warp] = v;
+        mean[warp][lane] = m;
+        lg[warp][lane] = valid ? log(m) : 0.0;
     }
     __syncthreads();
     double* out = scratch + scratch_off[pi] + (int64_t)slice * (S + 1);
-    for (int c = tid; c <= S; c += blockDim.x) {
-        double acc = 0.0;
-        for (int w = 0; w < kSliceSites / 32; ++w) acc += red[c][w];
-        out[c] = acc;
+    const double a = mean[0][lane], b = mean[1][lane];
+    for (int c = warp; c <= S; c += kLogsumWarps) {
+        double v;
+        if (c == 0) {
+            const double T = lg[0][lane] - lg[1][lane];
+            if (valid && terms && terms[pi]) terms[pi][i] = T;
+            v = valid ? T : 0.0;
+        } else {  // quotients, not products by reciprocals: equal shifts give exactly 0
+            v = valid ? Pd.num[i * S + c - 1] / a - Pd.den[i * S + c - 1] / b : 0.0;
+        }
+        v = warp_sum_xor(v);
+        if (lane == 0) out[c] = v;
     }
 }
 
-__global__ void __launch_bounds__(32) logsum_final_kernel(const ProbDev* __restrict__ probs,
-                                                          ProbResult* __restrict__ results,
-                                                          const double* __restrict__ scratch,
-                                                          const int64_t* __restrict__ scratch_off) {
-    const int pi = blockIdx.x, lane = threadIdx.x;
+// Warp w of a problem's CTA adds slices w, w + 8, ... of its lanes' columns, the
+// first warp the eight sums of each column in order.
+__global__ void __launch_bounds__(32 * kLogsumWarps) logsum_final_kernel(const ProbDev* __restrict__ probs,
+                                                                         ProbResult* __restrict__ results,
+                                                                         const double* __restrict__ scratch,
+                                                                         const int64_t* __restrict__ scratch_off) {
+    __shared__ double red[kLogsumWarps][kMaxS + 1];
+    const int pi = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const ProbDev& Pd = probs[pi];
     const int64_t D = Pd.n_terms;
     const int S = Pd.S;
     if (D <= 0 || S < 2) return;
     const int slices = (int)((D + kSliceSites - 1) / kSliceSites);
     const double* part = scratch + scratch_off[pi];
+    for (int c = lane; c <= S; c += 32) {
+        double sum = 0.0;
+        for (int sl = warp; sl < slices; sl += kLogsumWarps) sum += part[(int64_t)sl * (S + 1) + c];
+        red[warp][c] = sum;
+    }
+    __syncthreads();
+    if (warp != 0) return;
     double col[3] = {0.0, 0.0, 0.0};  // columns lane, lane + 32, lane + 64 (S + 1 <= 65)
     for (int k = 0; k < 3; ++k) {
         const int c = lane + 32 * k;
         if (c <= S)
-            for (int sl = 0; sl < slices; ++sl) col[k] += part[(int64_t)sl * (S + 1) + c];
+            for (int w = 0; w < kLogsumWarps; ++w) col[k] += red[w][c];
     }
-    double log_p = __shfl_sync(0xffffffffu, col[0], 0);
+    const double log_p = __shfl_sync(0xffffffffu, col[0], 0);
+    // sum of the squared shift columns: this lane's in order, then across lanes
     double ss = 0.0;
-    for (int c = 1; c <= S; ++c) {
-        const double l = __shfl_sync(0xffffffffu, col[c >> 5], c & 31);
-        ss += l * l;
+    for (int k = 0; k < 3; ++k) {
+        const int c = lane + 32 * k;
+        if (c >= 1 && c <= S) ss = fma(col[k], col[k], ss);
     }
+    ss = warp_sum_xor(ss);
     if (lane == 0) {
         ProbResult& R = Pd.res ? *Pd.res : results[pi];
         R.log_p = log_p;
@@ -1126,13 +1165,65 @@ cudaError_t launch_one(const GenzTile& tile, const ProbDev* probs, const ItemSrc
 
 }  // namespace
 
+// Built-in tile (measured on the 50x50 grid): mixed blocks of up to 32
+// variables run two points per lane (one vote per step for both), FP64 one.
+// Warps, mixed: 4 (above 21 variables 8 where they divide the shifts: S = 16, m =
+// 30 5.89 against 5.97 ms), but where 4 would leave more than a fifth of their
+// rounds idle (S = 5, 6, 9) 5 or 3 if those divide S (S = 5, m = 20: 1.34 against
+// 1.59 ms; S = 6 1.52 against 1.70; S = 10 stays at 4: 2.43 against 2.55 with 5;
+// idle warps of one CTA leave their issue slots to the others).  FP64: up to 8
+// with the units (shifts x lattice slices) spread evenly: its function tables take
+// 45 KB a CTA, so 16 resident warps want two CTAs of 8 (55.6 against 58.2 ms with
+// 4 at m = 20).  Shift groups
+// (a power of two, so S = 2^k splits evenly) until a launch has ~2048 CTA items,
+// never fewer shifts per item than warps (a warp without a unit idles); ~4096 items
+// for blocks of up to 16 variables, which fit more CTAs per SM.  A launch whose
+// units all fit the GPU's resident warps at once gives each warp one, up to 12 warps
+// a CTA: its time is one unit's chain of steps (100 terms, S = 10: call 0.239 ms in
+// groups of 4 warps, 0.192 so).
+// Blocks above 32 variables: 8 warps, one point per lane, every shift of a term in
+// one item, so the Cholesky of up to 64 variables is shared by the most work.
+GenzTile default_tile(bool mixed, int64_t total_sites, int max_S, int bucket, int sms) {
+    GenzTile t;
+    const int dmax = kDmaxBuckets[bucket];
+    t.slices = 0;
+    if (dmax > 32) {
+        t.warps = 8;
+        t.points = 1;
+        t.groups = 1;
+        return t;
+    }
+    const int per_shift = auto_slices(max_S, 1 << 20, mixed ? kModeFast : kModeFP64);
+    const int units = max_S * per_shift;
+    t.points = mixed ? 2 : 1;
+    if (total_sites * units <= (int64_t)sms * 16) {
+        t.groups = (units + 11) / 12;
+        t.warps = (max_S + t.groups - 1) / t.groups * per_shift;
+        return t;
+    }
+    if (!mixed) {
+        const int rounds = (units + 7) / 8;
+        t.warps = (units + rounds - 1) / rounds;
+    } else if (dmax > 21 && max_S % 8 == 0) {
+        t.warps = 8;
+    } else {
+        const int full = (max_S + 3) / 4 * 4;
+        t.warps = 5 * max_S >= 4 * full ? 4 : max_S % 5 == 0 ? 5 : max_S % 3 == 0 ? 3 : 4;
+    }
+    // small blocks fit more CTAs per SM: they want more items
+    const int64_t target = dmax <= 16 ? 4096 : 2048;
+    int g = 1;
+    while (g < max_S && (int64_t)g * total_sites < target && max_S / (2 * g) >= t.warps) g *= 2;
+    t.groups = g;
+    return t;
+}
+
 cudaError_t launch_genz(int bucket, bool mixed, const GenzTile& tile, const ProbDev* probs,
                         const int* seg_prefix, const int2* seg_base, int n_segs, int n_sites,
                         ProbResult* results, int* fallback_count, int2* fallback_items, int max_S,
                         int fb_capacity, cudaStream_t st) {
     if (n_sites <= 0) return cudaSuccess;
     GenzTile t = tile;
-    if (t.slices < 1) t.slices = 1;
     if (t.groups < 1) t.groups = 1;
     if (t.groups > max_S) t.groups = max_S;
     const int per_group = (max_S + t.groups - 1) / t.groups;
@@ -1173,7 +1264,8 @@ cudaError_t launch_genz_fallback(int max_bucket, const ProbDev* probs, const int
                                  const int2* fallback_items, int capacity, ProbResult* results,
                                  int max_S, cudaStream_t st) {
     if (capacity <= 0) return cudaSuccess;
-    GenzTile t{4, 1, 1, 1};
+    // 16 warps a term (8 above 32 variables): its shifts in four slices each
+    GenzTile t{16, 1, 0, 1};
     ItemSrc src{fallback_items, fallback_count, nullptr, nullptr, 0, capacity, 1, 0, 1, 0};
     if (max_bucket >= 7)  // blocks of more than 32 variables in the batch
         return launch_one<64, 1, kModeSafe>(t, probs, src, max_S, results, nullptr, nullptr, st);
@@ -1184,9 +1276,9 @@ cudaError_t launch_logsum(const ProbDev* probs, int n_probs, int max_slices, Pro
                           double* const* terms, double* scratch, const int64_t* scratch_off,
                           cudaStream_t st) {
     if (n_probs <= 0 || max_slices <= 0) return cudaSuccess;
-    logsum_partial_kernel<<<dim3(max_slices, n_probs), kSliceSites, 0, st>>>(probs, terms, scratch,
-                                                                          scratch_off);
-    logsum_final_kernel<<<n_probs, 32, 0, st>>>(probs, results, scratch, scratch_off);
+    logsum_partial_kernel<<<dim3(max_slices, n_probs), 32 * kLogsumWarps, 0, st>>>(probs, terms, scratch,
+                                                                               scratch_off);
+    logsum_final_kernel<<<n_probs, 32 * kLogsumWarps, 0, st>>>(probs, results, scratch, scratch_off);
     return cudaGetLastError();
 }
 

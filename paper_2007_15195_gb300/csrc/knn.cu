@@ -58,6 +58,27 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
     return v;
 }
 
+// The grid of a bounding box given as keys: max ~x, max ~y, max x, max y.
+__device__ __forceinline__ Grid box_grid(const unsigned long long (&k)[4], int gbits) {
+    const double xmin = ord_value(~k[0]), ymin = ord_value(~k[1]);
+    const double xmax = ord_value(k[2]), ymax = ord_value(k[3]);
+    const double ex = xmax - xmin, ey = ymax - ymin;
+    const double s = (ex > ey) ? ex : ey;
+    Grid g;
+    g.xmin = xmin;
+    g.ymin = ymin;
+    g.zero = !(s > 0.0);
+    g.c = g.zero ? 0.0 : 1073741824.0 / s;
+    g.shift = 30 - gbits;
+    g.G = 1 << gbits;
+    return g;
+}
+
+__device__ __forceinline__ int2 quantise(const Grid& g, double x, double y) {
+    if (g.zero) return make_int2(0, 0);
+    return make_int2((int)floor(__dmul_rn(__dsub_rn(x, g.xmin), g.c)), (int)floor(__dmul_rn(__dsub_rn(y, g.ymin), g.c)));
+}
+
 // Bounding box of the sites: maxima of the keys of x, y and of their
 // complements (the minima), warp shuffles, then one atomic a warp and quantity;
 // the last CTA to finish writes the grid.  box: four keys and a counter, all
@@ -83,18 +104,7 @@ __global__ void __launch_bounds__(256) bbox_kernel(const double* __restrict__ si
         __threadfence();
 #pragma unroll
         for (int q = 0; q < 4; ++q) k[q] = atomicMax(&box[q], 0ULL);
-        const double xmin = ord_value(~k[0]), ymin = ord_value(~k[1]);
-        const double xmax = ord_value(k[2]), ymax = ord_value(k[3]);
-        const double ex = xmax - xmin, ey = ymax - ymin;
-        const double s = (ex > ey) ? ex : ey;
-        Grid g;
-        g.xmin = xmin;
-        g.ymin = ymin;
-        g.zero = !(s > 0.0);
-        g.c = g.zero ? 0.0 : 1073741824.0 / s;
-        g.shift = 30 - gbits;
-        g.G = 1 << gbits;
-        *out = g;
+        *out = box_grid(k, gbits);
     }
 }
 
@@ -104,38 +114,43 @@ __global__ void quantize_kernel(const double* __restrict__ sites, int64_t D,
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= D) return;
     const Grid g = *grid;
-    int qx = 0, qy = 0;
-    if (!g.zero) {
-        qx = (int)floor(__dmul_rn(__dsub_rn(sites[2 * i], g.xmin), g.c));
-        qy = (int)floor(__dmul_rn(__dsub_rn(sites[2 * i + 1], g.ymin), g.c));
-    }
-    qxy[i] = make_int2(qx, qy);
-    const int cell = (qy >> g.shift) * (g.G + 1) + (qx >> g.shift);
+    const int2 q = quantise(g, sites[2 * i], sites[2 * i + 1]);
+    qxy[i] = q;
+    const int cell = (q.y >> g.shift) * (g.G + 1) + (q.x >> g.shift);
     atomicAdd(&counts[cell], 1);
 }
 
-// Exclusive scan of the cell counts (one CTA; the grid has at most 1025^2 cells).
-__global__ void scan_kernel(const int* __restrict__ counts, int n, int* __restrict__ offsets,
-                            int* __restrict__ cursor) {
-    __shared__ int part[1024];
-    const int t = threadIdx.x, T = blockDim.x;
-    const int per = (n + T - 1) / T;
-    const int lo = t * per, hi = min(n, lo + per);
+// Exclusive scan of the cell counts (one CTA of 1,024 threads; the grid has at
+// most 1025^2 cells): a run of cells a thread, the threads' sums by warp shuffles
+// (one thread adding the 1,024 sums took 16 of the kernel's 25 us).
+__global__ void __launch_bounds__(1024) scan_kernel(const int* __restrict__ counts, int n, int* __restrict__ offsets,
+                                                    int* __restrict__ cursor) {
+    __shared__ int part[32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int per = (n + 1023) / 1024;
+    const int lo = min(n, t * per), hi = min(n, lo + per);
     int s = 0;
     for (int i = lo; i < hi; ++i) s += counts[i];
-    part[t] = s;
+    int run = s;  // inclusive over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, run, o);
+        if (lane >= o) run += v;
+    }
+    if (lane == 31) part[warp] = run;
     __syncthreads();
-    if (t == 0) {
-        int run = 0;
-        for (int k = 0; k < T; ++k) {
-            const int v = part[k];
-            part[k] = run;
-            run += v;
+    if (warp == 0) {
+        int w = part[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += v;
         }
-        offsets[n] = run;
+        part[lane] = w;
     }
     __syncthreads();
-    int run = part[t];
+    run += (warp > 0 ? part[warp - 1] : 0) - s;  // exclusive
+    if (t == 0) offsets[n] = part[31];
     for (int i = lo; i < hi; ++i) {
         offsets[i] = run;
         cursor[i] = run;
@@ -526,19 +541,89 @@ cudaError_t build_cells(const double* sites, int64_t D, void* scratch, cudaStrea
     return cudaGetLastError();
 }
 
+// Up to kSmallMax sites, one CTA, a thread a site: bounding box and quantised
+// coordinates (to qxy) and, with ORDER, first the XY order (each site's rank
+// counts the smaller keys) and the gather of sites and thresholds.  Every search
+// of such a problem is by brute force, so the cell grid is not built: one launch
+// of 9 us in place of four to ten (100 sites: 35 us of kernels, and their gaps).
+static_assert(kSmallMax <= kBruteLimit, "small problems need no cell grid");
+
+template <bool ORDER>
+__global__ void __launch_bounds__((int)kSmallMax) small_kernel(const double* __restrict__ sites,
+                                                               const double* __restrict__ u, int D,
+                                                               int32_t* __restrict__ perm,
+                                                               double* __restrict__ sites_out,
+                                                               double* __restrict__ u_out, int2* __restrict__ qxy) {
+    __shared__ unsigned long long kx[kSmallMax], ky[kSmallMax];
+    __shared__ unsigned long long part[4][kSmallMax / 32];
+    __shared__ Grid grid;
+    const int i = threadIdx.x, lane = i & 31, warp = i >> 5, nw = blockDim.x >> 5;
+    const bool in = i < D;
+    const double x = in ? sites[2 * i] : 0.0, y = in ? sites[2 * i + 1] : 0.0;
+    const unsigned long long mx = ord_key(x), my = ord_key(y);
+    unsigned long long k[4] = {in ? ~mx : 0, in ? ~my : 0, in ? mx : 0, in ? my : 0};
+    if (ORDER && in) {
+        kx[i] = mx;
+        ky[i] = my;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        k[q] = warp_max_u64(k[q]);
+        if (lane == 0) part[q][warp] = k[q];
+    }
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) k[q] = warp_max_u64(lane < nw ? part[q][lane] : 0ULL);
+        if (lane == 0) grid = box_grid(k, 0);
+    }
+    int rank = i;
+    if (ORDER && in) {
+        rank = 0;
+        for (int j = 0; j < D; ++j) {
+            const unsigned long long xj = kx[j], yj = ky[j];
+            rank += (xj < mx) || (xj == mx && (yj < my || (yj == my && j < i)));
+        }
+        perm[rank] = i;
+        sites_out[2 * rank] = x;
+        sites_out[2 * rank + 1] = y;
+        if (u) u_out[rank] = u[i];
+    }
+    __syncthreads();
+    if (in) qxy[rank] = quantise(grid, x, y);
+}
+
+int small_threads(int64_t D) { return (int)((D + 31) / 32 * 32); }
+
+template <int K>
+void run_search(const Cells& c, int64_t D, int m, int group, int32_t* nbr, cudaStream_t st) {
+    const int blocks = (int)((D + kSearchWarps - 1) / kSearchWarps);
+    search_kernel<K><<<blocks, 32 * kSearchWarps, 0, st>>>(c.qxy, D, m, group, c.grid, c.offsets, c.cell_pts, nbr);
+}
+
+cudaError_t launch_order_small(const double* sites, const double* u, int64_t D, int32_t* perm, double* sites_out,
+                               double* u_out, void* scratch, cudaStream_t st) {
+    small_kernel<true><<<1, small_threads(D), 0, st>>>(sites, u, (int)D, perm, sites_out, u_out, (int2*)scratch);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_knn_small(int64_t D, int m, int32_t* nbr, void* scratch, cudaStream_t st) {
+    const Cells c{nullptr, (int2*)scratch, nullptr, nullptr};
+    m <= 32 ? run_search<1>(c, D, m, 0, nbr, st) : run_search<2>(c, D, m, 0, nbr, st);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_knn(const double* sites, int64_t D, int m, int32_t* nbr, void* scratch,
                        cudaStream_t st, int group) {
     if (D <= 0 || m <= 0) return cudaSuccess;
-    Cells c;
-    cudaError_t e = build_cells(sites, D, scratch, st, c);
-    if (e != cudaSuccess) return e;
-    const int blocks_s = (int)((D + kSearchWarps - 1) / kSearchWarps);
-    if (m <= 32)
-        search_kernel<1><<<blocks_s, 32 * kSearchWarps, 0, st>>>(c.qxy, D, m, group, c.grid, c.offsets,
-                                                                  c.cell_pts, nbr);
-    else
-        search_kernel<2><<<blocks_s, 32 * kSearchWarps, 0, st>>>(c.qxy, D, m, group, c.grid, c.offsets,
-                                                                  c.cell_pts, nbr);
+    Cells c{nullptr, (int2*)scratch, nullptr, nullptr};
+    if (D <= kSmallMax) {
+        small_kernel<false><<<1, small_threads(D), 0, st>>>(sites, nullptr, (int)D, nullptr, nullptr, nullptr, c.qxy);
+    } else {
+        const cudaError_t e = build_cells(sites, D, scratch, st, c);
+        if (e != cudaSuccess) return e;
+    }
+    m <= 32 ? run_search<1>(c, D, m, group, nbr, st) : run_search<2>(c, D, m, group, nbr, st);
     return cudaGetLastError();
 }
 

@@ -112,19 +112,8 @@ extern "C" int vecchia_log_cdf_noalloc(int device, void* cuda_stream, const doub
     const bool mixed = precision == VECCHIA_MIXED;
     constexpr int kDim = vk::kMaxDim;
 
-    // tile: the built-in rule of vecchia_log_cdf (mixed: two points per lane up
-    // to 32 variables, 8 warps above 21; power-of-two shift groups for ~2048
-    // CTA items (4096 up to 16 variables), never fewer shifts per item than
-    // warps; above 32 variables 8
-    // warps, one point, one group)
     const int bucket = vk::bucket_of(m + 1);
-    const int dmax = vk::kDmaxBuckets[bucket];
-    const int warps = (mixed && dmax > 21) ? 8 : 4;
-    int groups = 1;
-    const int64_t target = dmax <= 16 ? 4096 : 2048;
-    while (groups < S && (int64_t)groups * D < target && S / (2 * groups) >= warps) groups *= 2;
-    vk::GenzTile tile{warps, mixed ? 2 : 1, 1, groups};
-    if (dmax > 32) tile = vk::GenzTile{8, 1, 1, 1};
+    const vk::GenzTile tile = vk::default_tile(mixed, D, S, bucket, vk::device_sm_count(device));
 
     // scratch layout (every offset a multiple of 256 bytes)
     size_t off = 0;
@@ -139,7 +128,7 @@ extern "C" int vecchia_log_cdf_noalloc(int device, void* cuda_stream, const doub
     const size_t o_delta = take(sizeof(double) * vk::kMaxS * kDim);
     const size_t o_dfix = take(sizeof(uint32_t) * vk::kMaxS * kDim);
     const size_t o_fbc = take(sizeof(int));
-    const size_t fb_cap = mixed ? (size_t)D * groups + (size_t)vk::genz_items_slack(vk::device_sm_count(device)) : 1;
+    const size_t fb_cap = mixed ? (size_t)D * tile.groups + (size_t)vk::genz_items_slack(vk::device_sm_count(device)) : 1;
     const size_t o_fbi = take(sizeof(int2) * fb_cap);
     // parameter block, uploaded in one copy
     struct Params {

@@ -81,9 +81,12 @@ struct ProbResult {
 struct GenzTile {
     int warps;      // warps per CTA (1..16)
     int points;     // points per lane per pass (1, 2 or 4): template parameter
-    int slices;     // lattice slices per shift, spread over the CTA's warps
+    int slices;     // lattice slices per shift, spread over the CTA's warps (0: by each problem's S and N)
     int groups;     // shift groups per site, spread over CTAs (N x S split)
 };
+
+// The built-in launch shape for a bucket of a batch (genz.cu).
+GenzTile default_tile(bool mixed, int64_t total_sites, int max_S, int bucket, int sms);
 
 // ---------------- kernels' host launchers (genz.cu, knn.cu) ----------------
 
@@ -123,6 +126,12 @@ cudaError_t launch_init_results(ProbResult* results, int n, int* fallback_count,
 size_t knn_scratch_bytes(int64_t D);
 cudaError_t launch_knn(const double* sites, int64_t D, int m, int32_t* nbr, void* scratch,
                        cudaStream_t st, int group = 0);
+// XY order, gather and quantised coordinates of up to kSmallMax sites in one
+// launch, and the neighbour search on those coordinates (scratch as for launch_knn).
+constexpr int64_t kSmallMax = 512;
+cudaError_t launch_order_small(const double* sites, const double* u, int64_t D, int32_t* perm, double* sites_out,
+                               double* u_out, void* scratch, cudaStream_t st);
+cudaError_t launch_knn_small(int64_t D, int m, int32_t* nbr, void* scratch, cudaStream_t st);
 // Exact maxmin ordering on the device (one thread-block cluster); perm (D, device)
 // gets new position -> old index; scratch from maxmin_scratch_bytes(D).
 size_t maxmin_scratch_bytes(int64_t D);
@@ -194,6 +203,15 @@ cudaError_t launch_full_genz_tc(const double* A, const double* u, int64_t D, int
                                 const uint32_t* dfix, int dim, void* scratch, double* part, int* timeout,
                                 uint64_t wait_ns, int withhold, cudaEvent_t ev_begin, cudaEvent_t ev_end,
                                 cudaStream_t st);
+
+// The FP64 recursion with its contraction on the tensor cores (full_fix_tc.cu),
+// given the FP64 factor A: part gets part_stride sums per shift, of which it
+// writes the first ceil(N / 128) (the caller zeroes the rest).
+size_t full_fix_tc_scratch_bytes(int64_t D, int64_t N, int S);
+cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int64_t N, int S, const uint32_t* g,
+                               const double* delta, int dim, void* scratch, double* part, int part_stride,
+                               int* timeout, uint64_t wait_ns, cudaEvent_t ev_begin, cudaEvent_t ev_end,
+                               cudaStream_t st);
 
 // sites_out[k] = sites[perm[k]], u_out[k] = u[perm[k]]; *bad = 1 on an index out of range.
 cudaError_t launch_gather(const int32_t* perm, const double* sites, const double* u, int64_t D,
