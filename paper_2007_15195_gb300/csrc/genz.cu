@@ -1171,10 +1171,10 @@ cudaError_t launch_one(const GenzTile& tile, const ProbDev* probs, const ItemSrc
 // 30 5.89 against 5.97 ms), but where 4 would leave more than a fifth of their
 // rounds idle (S = 5, 6, 9) 5 or 3 if those divide S (S = 5, m = 20: 1.34 against
 // 1.59 ms; S = 6 1.52 against 1.70; S = 10 stays at 4: 2.43 against 2.55 with 5;
-// idle warps of one CTA leave their issue slots to the others).  FP64: up to 8
-// with the units (shifts x lattice slices) spread evenly: its function tables take
-// 45 KB a CTA, so 16 resident warps want two CTAs of 8 (55.6 against 58.2 ms with
-// 4 at m = 20).  Shift groups
+// idle warps of one CTA leave their issue slots to the others).  FP64: of 8 down to 4
+// what keeps the most warps at work, 16 resident and the units (shifts x lattice
+// slices) in rounds of w: 8 for S = 16 (55.6 against 58.2 ms with 4 at m = 20),
+// 4 for 12 units (S = 6, 333 terms: 0.68 against 0.77 ms with 6).  Shift groups
 // (a power of two, so S = 2^k splits evenly) until a launch has ~2048 CTA items,
 // never fewer shifts per item than warps (a warp without a unit idles); ~4096 items
 // for blocks of up to 16 variables, which fit more CTAs per SM.  A launch whose
@@ -1202,8 +1202,14 @@ GenzTile default_tile(bool mixed, int64_t total_sites, int max_S, int bucket, in
         return t;
     }
     if (!mixed) {
-        const int rounds = (units + 7) / 8;
-        t.warps = (units + rounds - 1) / rounds;
+        double best = 0.0;
+        for (int w = 8; w >= 4; --w) {
+            const double rate = (double)(16 / w * w) * units / (w * ((units + w - 1) / w));
+            if (rate > 1.001 * best) {
+                best = rate;
+                t.warps = w;
+            }
+        }
     } else if (dmax > 21 && max_S % 8 == 0) {
         t.warps = 8;
     } else {
