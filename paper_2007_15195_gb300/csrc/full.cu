@@ -361,8 +361,9 @@ struct FullSmem {
 // contraction (four warps, 16 independent products a thread and variable).
 // The contraction's D^2/2 products a point cost 25 cycles a warp instruction
 // triple against the FP64 fma's 76.  (Tiles of 128 points left 152 SMs with 1 or 2
-// tiles each at N S = 24,000.)  D = 1,021, N S = 24,000: 52.2 -> 13.4 ms a call
-// (2.7 ms of it the factor); D = 2,500, N S = 65,536: 501 -> 145 ms.
+// tiles each at N S = 24,000.)  D = 1,021, N S = 24,000: 10.6 ms, D = 2,500, N S =
+// 65,536: 134 ms (490 in FP64); the tensor-core form takes 3.8 and 38 ms, so this one serves the
+// smallest problems and histories beyond kFixTcMaxBytes.
 __global__ void __launch_bounds__(kFullThreads) full_genz_kernel(const fix::Digits* __restrict__ Ld,
                                                                  const FixVar* __restrict__ var, FullArgs a,
                                                                  fix::Digits* __restrict__ Y,
@@ -746,6 +747,16 @@ int64_t full_genz_blocks_per_shift(int64_t N, bool mixed) {
 
 // Scratch: the shared part (factor, lattice and shift tables, block sums,
 // status words) followed by the precision's own tables and y history.
+// FP64 recursion: the tensor cores' contraction from kFixTcMin variables on (N S =
+// 24,000: D = 64 0.13 against 0.16 ms, D = 256 0.54 against 0.94, D = 1,021 3.8
+// against 10.6), unless its history (16 bytes a y value, twice the integer form's)
+// would not fit beside other work.
+constexpr int64_t kFixTcMin = 64;
+constexpr size_t kFixTcMaxBytes = 96ull << 30;
+bool fix_tc_pays(int64_t D, int64_t N, int S) {
+    return D >= kFixTcMin && full_fix_tc_scratch_bytes(D, N, S) <= kFixTcMaxBytes;
+}
+
 size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed) {
     const int64_t bps = (N + kFullP - 1) / kFullP, nblk = full_genz_blocks_per_shift(N, mixed);
     const int64_t dim = D > 1 ? D - 1 : 1;
@@ -754,6 +765,7 @@ size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed) {
                           al(sizeof(uint32_t) * S * dim) + al(sizeof(double) * S * nblk) + al(2 * sizeof(int)) +
                           al(sizeof(uint64_t) + 2 * sizeof(int64_t) + sizeof(int32_t));
     if (mixed) return shared + al(chol_tc_scratch_bytes(D)) + full_tc_scratch_bytes(D, N, S);
+    if (fix_tc_pays(D, N, S)) return shared + full_fix_tc_scratch_bytes(D, N, S);
     return shared + al(sizeof(fix::Digits) * D * D) + al(sizeof(FixVar) * D) +
            al(sizeof(fix::Digits) * (size_t)S * bps * D * kFullP);
 }
@@ -807,6 +819,11 @@ cudaError_t launch_full_genz(const double* sites, const double* u, int64_t D, co
     if (mixed) {
         e = launch_full_genz_tc(A, u, D, N, S, gdev + dim, dfix, (int)dim, p, part, bad + 1, wait_ns, withhold,
                                 ev_begin, ev_end, st);
+    } else if (fix_tc_pays(D, N, S)) {
+        e = cudaMemsetAsync(part, 0, sizeof(double) * S * nblk, st);
+        if (e == cudaSuccess)
+            e = launch_full_fix_tc(A, u, D, N, S, gdev, delta, (int)dim, p, part, (int)nblk, bad + 1, wait_ns, ev_begin,
+                                   ev_end, st);
     } else {
         void* Ld = p;
         p += al(sizeof(fix::Digits) * D * D);

@@ -204,6 +204,15 @@ cudaError_t launch_full_genz_tc(const double* A, const double* u, int64_t D, int
                                 uint64_t wait_ns, int withhold, cudaEvent_t ev_begin, cudaEvent_t ev_end,
                                 cudaStream_t st);
 
+// The FP64 recursion with its contraction on the tensor cores (full_fix_tc.cu),
+// given the FP64 factor A: part gets part_stride sums per shift, of which it
+// writes the first ceil(N / 128) (the caller zeroes the rest).
+size_t full_fix_tc_scratch_bytes(int64_t D, int64_t N, int S);
+cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int64_t N, int S, const uint32_t* g,
+                               const double* delta, int dim, void* scratch, double* part, int part_stride,
+                               int* timeout, uint64_t wait_ns, cudaEvent_t ev_begin, cudaEvent_t ev_end,
+                               cudaStream_t st);
+
 // sites_out[k] = sites[perm[k]], u_out[k] = u[perm[k]]; *bad = 1 on an index out of range.
 cudaError_t launch_gather(const int32_t* perm, const double* sites, const double* u, int64_t D,
                           double* sites_out, double* u_out, int* bad, cudaStream_t st);
