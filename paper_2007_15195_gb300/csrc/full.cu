@@ -160,43 +160,41 @@ __global__ void __launch_bounds__(512) chol_diag_kernel(double* __restrict__ A, 
     }
 }
 
-// Rows r >= k0 + 32 of the block column: x L_kk^T = a by forward
-// substitution, one thread per row, blockDim.x (8 to 32) rows per CTA.  The
-// solve is right-looking: once x_j is known it goes into every later
-// accumulator, so each x_k still receives its terms in ascending j with fma
-// (bit for bit the row-by-row definition's sums).  Each entry divides by its
+// Rows r >= k0 + 32 of the block column: x L_kk^T = a by forward substitution, one
+// warp per row, lane j holding x_j.  Once x_j is known it goes into every later
+// lane's accumulator, so each x_k still receives its terms in ascending j with
+// fma (bit for bit the row-by-row definition's sums), and each entry is divided by its
 // pivot (the definition's operation: a reciprocal would change the factor's
-// last bits, and with them which exactly singular block is reported).
-__global__ void chol_trsm_kernel(double* __restrict__ A, int D, int k0) {
-    __shared__ double Lk[kCholB][kCholB + 1];
+// last bits, and with them which exactly singular block is reported; exact_math.h).
+// Two warp instructions on the FP64 pipe a column instead of a thread's 528 fma:
+// 7 against 41 us a block column at D = 1,021.
+constexpr int kTrsmWarps = 4;
+__global__ void __launch_bounds__(32 * kTrsmWarps) chol_trsm_kernel(double* __restrict__ A, int D, int k0) {
+    __shared__ double T[kCholB][kCholB + 1];
     __shared__ exact::Pivot piv[kCholB];
-    // the diagonal block, a row per thread and pass with its 32 loads issued
-    // together (a CTA has as few as 8 threads: a load loop would wait on L2
-    // 128 times in sequence)
-    for (int r = threadIdx.x; r < kCholB; r += blockDim.x) {
-        const double* src = A + (int64_t)(k0 + r) * D + k0;
-        double v[kCholB];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    {  // the factored diagonal block: 8 loads a thread, issued together
+        const int r = tid >> 2, c0 = (tid & 3) * 8;
+        const double* src = A + (int64_t)(k0 + r) * D + k0 + c0;
+        double v[8];
 #pragma unroll
-        for (int c = 0; c < kCholB; ++c) v[c] = (c <= r) ? src[c] : 0.0;
+        for (int c = 0; c < 8; ++c) v[c] = (c0 + c <= r) ? src[c] : 0.0;
 #pragma unroll
-        for (int c = 0; c < kCholB; ++c) Lk[r][c] = v[c];
-        piv[r] = exact::pivot_of(Lk[r][r]);
+        for (int c = 0; c < 8; ++c) T[r][c0 + c] = v[c];
     }
     __syncthreads();
-    const int r = k0 + kCholB + blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= D) return;
+    if (tid < kCholB) piv[tid] = exact::pivot_of(T[tid][tid]);
+    __syncthreads();
+    const int r = k0 + kCholB + blockIdx.x * kTrsmWarps + warp;
+    if (r >= D) return;  // warp-uniform
     double* row = A + (int64_t)r * D + k0;
-    double x[kCholB];
-#pragma unroll
-    for (int j = 0; j < kCholB; ++j) x[j] = row[j];
-#pragma unroll
+    double acc = row[lane];
     for (int j = 0; j < kCholB; ++j) {
-        x[j] = exact::quotient(x[j], piv[j]);
-#pragma unroll
-        for (int k = j + 1; k < kCholB; ++k) x[k] = fma(-x[j], Lk[k][j], x[k]);
+        if (lane == j) acc = exact::quotient(acc, piv[j]);
+        const double xj = __shfl_sync(0xffffffffu, acc, j);
+        if (lane > j) acc = fma(-xj, T[lane][j], acc);
     }
-#pragma unroll
-    for (int j = 0; j < kCholB; ++j) row[j] = x[j];
+    row[lane] = acc;
 }
 
 // Rows r >= k0 + 32 of the block column for the mixed path, whose trailing
@@ -504,11 +502,10 @@ cudaError_t launch_full_genz_fix(const double* A, const double* u, const FullArg
 
 }  // namespace
 
-// Rows per CTA of the row solve: 32 while that still gives every SM a CTA,
-// else fewer (down to 8), so the solve of a block column uses as many of the
-// SMs' FP64 units as its rows allow.
-int trsm_rows_per_cta(int64_t rows, int64_t sms) {
-    return rows >= 32 * sms ? 32 : rows >= 16 * sms ? 16 : 8;
+// Row solve of block column k0 (a warp a row).
+void launch_trsm(double* A, int64_t D, int64_t k0, cudaStream_t st) {
+    const int64_t rows = D - k0 - kCholB;
+    chol_trsm_kernel<<<(unsigned)((rows + kTrsmWarps - 1) / kTrsmWarps), 32 * kTrsmWarps, 0, st>>>(A, (int)D, (int)k0);
 }
 
 // Blocked Cholesky with a one-block lookahead on two streams.  The caller's
@@ -550,7 +547,7 @@ struct CholStreams {
 
 // The blocked factor of the covariance in A (see launch_cov_chol), queued on st.
 cudaError_t enqueue_chol(double* A, int64_t D, int* bad, cudaStream_t st, void* tc_scratch, int* timeout,
-                         uint64_t wait_ns, int64_t sms, CholStreams& cs) {
+                         uint64_t wait_ns, CholStreams& cs) {
     cudaError_t e = cudaSuccess;
     const int64_t nblk = (D + kCholB - 1) / kCholB;
     if (nblk <= 2 || e != cudaSuccess) {  // nothing to overlap
@@ -558,8 +555,7 @@ cudaError_t enqueue_chol(double* A, int64_t D, int* bad, cudaStream_t st, void* 
             chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, (int)k0, bad, 0);
             const int64_t rows = D - k0 - kCholB;
             if (rows > 0) {
-                const int rb = trsm_rows_per_cta(rows, sms);
-                chol_trsm_kernel<<<(unsigned)((rows + rb - 1) / rb), rb, 0, st>>>(A, (int)D, (int)k0);
+                launch_trsm(A, D, k0, st);
                 chol_update_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(A, (int)D, (int)k0, 0);
             }
             e = cudaGetLastError();
@@ -629,8 +625,7 @@ cudaError_t enqueue_chol(double* A, int64_t D, int* bad, cudaStream_t st, void* 
             e = cudaGetLastError();
             break;
         }
-        const int rb = trsm_rows_per_cta(rows, sms);
-        chol_trsm_kernel<<<(unsigned)((rows + rb - 1) / rb), rb, 0, st>>>(A, (int)D, (int)k0);
+        launch_trsm(A, D, k0, st);
         const int64_t tiles = (rows + kCholB - 1) / kCholB;
         if (tiles > 1) {  // the rest of step k on the side stream
             if (e == cudaSuccess) e = cudaEventRecord(ev_panel, st);
@@ -687,7 +682,6 @@ cudaError_t launch_cov_chol(const double* sites, int64_t D, const vecchia_cov& c
     if (D <= 0) return cudaSuccess;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
-    const int64_t sms = device_sm_count(dev);
     full_cov_kernel<<<dim3((unsigned)((D + 127) / 128), (unsigned)D), 128, 0, st>>>(sites, (int)D, cov_params(cov), A);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -711,14 +705,14 @@ cudaError_t launch_cov_chol(const double* sites, int64_t D, const vecchia_cov& c
     CholStreams cs;
     e = cs.create(tc);
     if (e != cudaSuccess) return e;
-    if (!graph) return enqueue_chol(A, D, bad, st, tc_scratch, timeout, wait_ns, sms, cs);
+    if (!graph) return enqueue_chol(A, D, bad, st, tc_scratch, timeout, wait_ns, cs);
     cudaGraph_t g = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaStream_t cap = nullptr;  // capture only: nothing runs on it
     e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        const cudaError_t eq = enqueue_chol(A, D, bad, cap, tc_scratch, timeout, wait_ns, sms, cs);
+        const cudaError_t eq = enqueue_chol(A, D, bad, cap, tc_scratch, timeout, wait_ns, cs);
         e = cudaStreamEndCapture(cap, &g);
         if (eq != cudaSuccess) e = eq;
     }
@@ -728,7 +722,7 @@ cudaError_t launch_cov_chol(const double* sites, int64_t D, const vecchia_cov& c
     if (e != cudaSuccess) {  // not capturable here: queue it eagerly
         cudaGetLastError();
         if (exec) cudaGraphExecDestroy(exec);
-        return enqueue_chol(A, D, bad, st, tc_scratch, timeout, wait_ns, sms, cs);
+        return enqueue_chol(A, D, bad, st, tc_scratch, timeout, wait_ns, cs);
     }
     {
         std::lock_guard<std::mutex> lk(g_chol_mu);
