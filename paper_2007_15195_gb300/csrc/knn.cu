@@ -341,28 +341,38 @@ __global__ void __launch_bounds__(32 * kSearchWarps) search_kernel(
         const int G = g.G, W = G + 1;
         const long long cs = 1LL << g.shift;
         const int cx0 = me.x >> g.shift, cy0 = me.y >> g.shift;
-        for (int r = 0;; ++r) {
-            for (int cy = cy0 - r; cy <= cy0 + r; ++cy) {
-                if (cy < 0 || cy > G) continue;
-                const bool edge_row = (cy == cy0 - r) || (cy == cy0 + r);
-                const int step = (edge_row || r == 0) ? 1 : 2 * r;
-                for (int cxx = cx0 - r; cxx <= cx0 + r; cxx += step) {
-                    if (cxx < 0 || cxx > G) continue;
-                    const int cell = cy * W + cxx;
-                    const int b = offsets[cell], e = offsets[cell + 1];
-                    for (int base = b; base < e; base += 32) {
-                        const int p = base + lane;
-                        Key k = inf_key();
-                        bool valid = false;
-                        if (p < e) {
-                            const int4 o = cell_pts[p];
-                            valid = o.z < lim;
-                            k.d2 = qdist2(me.x, me.y, o.x, o.y);
-                            k.j = o.z;
-                        }
-                        offer(valid, k);
-                    }
+        // the sites of cells [xa, xb] of row cy (contiguous in cell_pts)
+        auto cells = [&](int cy, int xa, int xb) {
+            xa = max(xa, 0);
+            xb = min(xb, G);
+            if (cy < 0 || cy > G || xa > xb) return;
+            const int b = offsets[cy * W + xa], e = offsets[cy * W + xb + 1];
+            for (int base = b; base < e; base += 32) {
+                const int p = base + lane;
+                Key k = inf_key();
+                bool valid = false;
+                if (p < e) {
+                    const int4 o = cell_pts[p];
+                    valid = o.z < lim;
+                    k.d2 = qdist2(me.x, me.y, o.x, o.y);
+                    k.j = o.z;
                 }
+                offer(valid, k);
+            }
+        };
+        // rings 0 and 1 together (few cells hold q sites, and a merge of a part
+        // chunk costs as much as a full one), then ring by ring, each row of cells as
+        // one run of candidates (100,000 sites in maxmin order, m = 30: 657 -> 400 us)
+        for (int r = 1;; ++r) {
+            if (r == 1) {
+                for (int cy = cy0 - 1; cy <= cy0 + 1; ++cy) cells(cy, cx0 - 1, cx0 + 1);
+            } else {
+                cells(cy0 - r, cx0 - r, cx0 + r);
+                for (int cy = cy0 - r + 1; cy < cy0 + r; ++cy) {
+                    cells(cy, cx0 - r, cx0 - r);
+                    cells(cy, cx0 + r, cx0 + r);
+                }
+                cells(cy0 + r, cx0 - r, cx0 + r);
             }
             flush();
             const Key w = worst();
@@ -786,7 +796,7 @@ cudaError_t launch_sort(KEYS keys, int64_t D, int32_t* perm, void* scratch, cuda
 // 0.47 -> 0.16 ms; 8,000 sites crowded about a point 127 -> 16 ms.
 
 constexpr int kMmThreads = 1024;
-constexpr int kMmSerial = 32;
+constexpr int kMmSerial = 32;  // (D = 100,000: 1.07 ms with 16, 0.96 with 32, 1.05 with 64)
 constexpr int kMmMaxCluster = 16;
 constexpr int kMmRounds = 16;        // grid-wide rounds
 constexpr int64_t kMmGridWide = 6000;  // from this many sites on
