@@ -69,10 +69,10 @@ SM_COUNT = 152          # replaced by the device's SM count (init_peaks)
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ = 2070.0     # replaced by the measured maximum SM clock (init_peaks)
 PEAK_SOURCE = "GB300 nominal: 152 SMs, 2070 MHz"
-# FP64 lanes per SM (an FMA counting once): GB300's FP64 rate is 1/64 of its
-# FP32 rate (1.25 TFLOP/s FP64 nominal = 152 SMs x 2 FMA lanes x 2 flops x
-# 2.07 GHz).
-FP64_LANES_PER_SM = 2
+# 64-bit products (the high half of 64 x 64 bits: three 32 x 32 + 64-bit
+# multiply-adds) per SM and clock: a multiply-add takes 4 cycles a warp and SMSP
+# (microbenchmark), so 4 SMSPs x 32 lanes / (3 x 4).
+FIX_PRODUCTS_PER_SM = 32.0 / 3.0
 ALG_OPS_STEP = 31
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of
 # the Genz kernel on the headline workload (m = 20, built-in tile:
@@ -85,7 +85,7 @@ GENZ_NCU_M20 = {"fma_pipe_active": 0.566, "issue_active": 0.773, "inst_per_step"
                 "source": "ncu --set full of one genz_kernel<21, 2, 1> launch of this workload"}
 # DRAM bytes of one launch of the FP64 Genz kernel on the headline workload
 # (genz_kernel<21, 1, FP64>), from one ncu capture of that launch.
-GENZ64_TRAFFIC_BYTES_M20 = 497_408
+GENZ64_TRAFFIC_BYTES_M20 = 454_912
 # DRAM bytes of one launch of the full-Genz recursion kernel on the tensor
 # cores (full_genz_tc_kernel, 50x50 grid, D = 2,500, N = 4,096 x S = 16), from
 # one ncu capture of that launch: 13.26 GB read + 1.56 GB written.
@@ -127,8 +127,8 @@ def fp32_peak():
 
 
 def fp64_peak():
-    """FP64 lane operations per second (an FMA counting once)."""
-    return SM_COUNT * FP64_LANES_PER_SM * SM_MAX_MHZ * 1e6
+    """64-bit fixed-point products per second."""
+    return SM_COUNT * FIX_PRODUCTS_PER_SM * SM_MAX_MHZ * 1e6
 
 
 def hbm_peak_gbs():
@@ -198,19 +198,14 @@ def alu_roofline(work_ops, seconds, kernel, note=None):
     return r
 
 
-# FP64-pipe roofline of the FP64 Genz kernel: FP64 operations per Genz step of
-# the formulation the kernel evaluates (an FMA counting once) -- running
-# product 1, lattice-weighted probabilities 2, Phi^{-1} 30 (Phi(-a0) and
-# phi(a0) at the first guess 24: interval map 2, degree-8 polynomial 8, a^2
-# as hi + lo 2, exponential 10, products 2; residual, quotient with one
-# correction and Halley factor 6), standardisation 1, Phi 24 (Phi(-|z|) 23,
-# 1 - T 1) -- plus (t + 1) FMAs for the conditional mean of row t + 1.
-# Compares, min/max, selects, powers of two and the integer lattice and
-# exponent work are not counted (the kernel does them with integer
-# instructions).
-FP64_OPS_STEP = 58
-FP64_OPS_NOTE = ("FP64-pipe lane operations, an FMA counting once; 58 per Genz step + q(q+1)/2 FMAs per "
-                 "point; peak = SMs x 2 FP64 lanes x max SM clock")
+# Roofline of the FP64 Genz kernel, which evaluates the step in 64-bit fixed
+# point: 64-bit products per Genz step -- lattice-weighted probability 1, the
+# polynomials of Phi^{-1} and Phi 3 each (their upper terms are 32-bit),
+# standardisation 1, running product 1 -- plus t + 1 for the conditional mean of
+# row t + 1.  Additions, shifts, selects and table indices are not counted.
+FP64_OPS_STEP = 9
+FP64_OPS_NOTE = ("64-bit fixed-point products (three 32 x 32 + 64-bit multiply-adds each); 9 per Genz step + "
+                 "q(q+1)/2 per point; peak = SMs x 32/3 products per clock x max SM clock")
 
 
 def fp64_alg_ops_q(q, N, S):
@@ -469,11 +464,11 @@ def run_ours(args):
                     "p99_ms": float(np.percentile(ms64, 99)), "genz_kernel_ms": g64 * 1000.0}
         if w64 is not None:
             fp64_obj["roofline"] = {"bound": "alu", "achieved": w64 / g64 / 1e12, "peak": fp64_peak() / 1e12,
-                                    "unit": "TFLOP/s", "frac": w64 / g64 / fp64_peak(),
+                                    "unit": "Tproduct/s", "frac": w64 / g64 / fp64_peak(),
                                     "traffic": GENZ64_TRAFFIC_BYTES_M20 if m == 20 else None,
                                     "kernel": "genz_kernel (fp64)", "kernel_ms": g64 * 1000.0,
-                                    "peak_source": "%d SMs x %d FP64 lanes x %.0f MHz (%s)"
-                                                   % (SM_COUNT, FP64_LANES_PER_SM, SM_MAX_MHZ, PEAK_SOURCE),
+                                    "peak_source": "%d SMs x %.2f products/clk x %.0f MHz (%s)"
+                                                   % (SM_COUNT, FIX_PRODUCTS_PER_SM, SM_MAX_MHZ, PEAK_SOURCE),
                                     "ops": FP64_OPS_NOTE}
 
     line = {"metric": metric_for(args.m), "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -865,7 +860,7 @@ def measure_large(args, compact=False):
                            "genz_kernel_s": g64,
                            "roofline": None if w64 is None else
                                        {"bound": "alu", "achieved": w64 / g64 / 1e12, "peak": fp64_peak() / 1e12,
-                                        "unit": "TFLOP/s", "frac": w64 / g64 / fp64_peak(), "traffic": None,
+                                        "unit": "Tproduct/s", "frac": w64 / g64 / fp64_peak(), "traffic": None,
                                         "kernel": "genz_kernel (fp64)", "ops": FP64_OPS_NOTE},
                            "mixed_vs_fp64": {"abs": abs(lpm - lp64), "tol": 1e-4 * max(1.0, abs(lp64)),
                                              "max_abs_dterm": float(d.max()), "by_conditioning": bins,
