@@ -71,9 +71,10 @@ __device__ __forceinline__ void pair_table(unsigned short* tab) {
 // (exact_math.h: the same values as the FP64 square root and division by a
 // shorter chain of integer instructions), then the packed trailing triangle
 // takes one fma per entry, spread over the threads through the pair table.
-// Warp 0 updates the next column first and goes on to its pivot while the other
-// warps take the rest, so a step costs warp 0's chain and one barrier.  Returns
-// the first non-positive pivot, or -1.
+// Warp 0 updates the next column first and goes on to its pivot while the warps of
+// the other three SMSPs take the rest (an FP64 instruction holds its SMSP's pipe for
+// 76 cycles, and warp 0's would queue behind theirs), so a step costs warp 0's
+// chain and one barrier.  Returns the first non-positive pivot, or -1.
 __device__ int factor_block(double (*T)[kCholB + 1], const unsigned short* tab, int b) {
     const int tid = threadIdx.x;
     for (int j = 0; j < b; ++j) {
@@ -93,9 +94,10 @@ __device__ int factor_block(double (*T)[kCholB + 1], const unsigned short* tab, 
         if (tid < 32) {
             if (tid < b - 1 - j) T[j + 1 + tid][j + 1] = fma(-T[j + 1 + tid][j], T[j + 1][j], T[j + 1 + tid][j + 1]);
             __syncwarp();
-        } else {
-            const int n = b - 2 - j;
-            for (int e = tid - 32; e < n * (n + 1) / 2; e += blockDim.x - 32) {
+        } else if ((tid >> 5) & 3) {
+            const int n = b - 2 - j, w = tid >> 5;
+            for (int e = ((w >> 2) * 3 + (w & 3) - 1) * 32 + (tid & 31); e < n * (n + 1) / 2;
+                 e += (int)blockDim.x / 4 * 3) {
                 const unsigned t = tab[e];
                 const int r = j + 2 + (int)(t >> 8), cc = j + 2 + (int)(t & 255u);
                 T[r][cc] = fma(-T[r][j], T[cc][j], T[r][cc]);

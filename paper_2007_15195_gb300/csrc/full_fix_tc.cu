@@ -19,11 +19,11 @@
 // A CTA takes 128 lattice points (MMA rows).  Four warps, one thread a point, run the
 // panels: they add the accumulators of each group of 128 variables to the points'
 // sums in shared memory, run the panel's variables in order, and write their y
-// as digits to the history.  A fifth warp's lane streams history chunks of 16
+// as digits to the history.  One lane of a fifth warp streams history chunks of 16
 // variables (32 KB of y digits, 8 KB of the panel's L digits) with cp.async.bulk
-// through a three-stage ring and issues 36 MMAs (M = 128, N = 32, K = 16) a chunk.
-// Two sets of accumulators (2 x 8 x 32 columns) alternate between groups, so it
-// runs up to two groups ahead, into the next panel during the points' pass; only
+// through a three-stage ring; one lane of a sixth issues 36 MMAs (M = 128, N = 32, K = 16)
+// a chunk.  Two sets of accumulators (2 x 8 x 32 columns) alternate between groups, so they
+// run up to two groups ahead, into the next panel during the points' pass; only
 // the chunks of that pass wait for it.  Operands lie in no-swizzle K-major core matrices
 // (8 rows x 16 bytes): per group of 8 rows the eight digit matrices of a chunk,
 // 256 bytes each (K stride 128 bytes, row-group stride 2,048).  Every wait is bounded by
@@ -50,7 +50,7 @@ constexpr int kXK = 16;        // history chunk (variables) = MMA K
 constexpr int kXDig = 8;       // digits
 constexpr int kXGroup = 8;     // chunks per accumulation
 constexpr int kXStages = 3;
-constexpr int kXThreads = kXP + 32;
+constexpr int kXThreads = kXP + 64;  // point warps, the MMA warp, the copy warp
 constexpr uint32_t kRowGroup = kXDig * 256;               // 8 rows: eight 256-byte digit matrices
 constexpr uint32_t kXChunkA = (kXP / 8) * kRowGroup;      // 32,768
 constexpr uint32_t kXChunkB = (kXB / 8) * kRowGroup;      // 8,192
@@ -230,54 +230,49 @@ __global__ void __launch_bounds__(128) fix_tc_tables_kernel(const double* __rest
             (v < D && v0 + tid < v) ? fix_coef(row[v0 + tid], kL) : fix::Digits{0, 0};
 }
 
-// The copies and MMAs of every panel, by one lane: chunk c < 2 p of panel p.
-__device__ void issue_all(const XArgs& a, XSmem& sm, const unsigned char* Yt) {
-    const int total = a.nP * (a.nP - 1);
+__device__ void give_up(const XArgs& a, XSmem& sm) {
+    atomicExch(&sm.abort, 1);
+    atomicExch(a.timeout, 1);
+}
+
+// The copies of every panel, by one lane of its own (a lane that also issued the
+// MMAs refilled a stage only after the next chunk's wait): chunk c < 2 p of panel p
+// once the points have written the panel that it holds and its stage is free.
+__device__ void copy_all(const XArgs& a, XSmem& sm, const unsigned char* Yt) {
+    int il = 0, seen = 0;  // copies issued; panels whose y the points have written
+    bool ok = true;
+    for (int p = 1; p < a.nP && ok; ++p)
+        for (int c = 0; c < 2 * p && ok; ++c) {
+            while (ok && seen <= c / 2) {
+                ok = mbar_wait(&sm.ydone, (uint32_t)(seen & 1), a.wait_ns, &sm.abort);
+                ++seen;
+            }
+            const int st = il % kXStages;
+            ok = ok && mbar_wait(&sm.empty[st], (uint32_t)(((il / kXStages) & 1) ^ 1), a.wait_ns, &sm.abort);
+            if (!ok) break;
+            mbar_expect_tx(&sm.full[st], kXStage);
+            bulk_g2s(sm.stage[st], Yt + (int64_t)c * kXChunkA, kXChunkA, &sm.full[st]);
+            bulk_g2s(sm.stage[st] + kXChunkA, a.Lb + ((int64_t)p * a.nC + c) * kXChunkB, kXChunkB, &sm.full[st]);
+            ++il;
+        }
+    if (!ok) give_up(a, sm);
+    // the copies in flight, bounded
+    for (int i = max(0, il - kXStages); i < il; ++i)
+        mbar_wait(&sm.full[i % kXStages], (uint32_t)((i / kXStages) & 1), kXWaitNs, nullptr);
+}
+
+// The MMAs of every panel, by one lane.
+__device__ void mma_all(const XArgs& a, XSmem& sm) {
     const uint32_t tmem = sm.tmem;
-    int il = 0, lp = 1, lc = 0;      // next load: panel, chunk
-    int seen = 0;                    // panels whose y the points have written
-    int groups = 0;                  // accumulations issued
-    bool failed = false;
-    // wait: block for the stage and the points' y; else only if both are there
-    auto load = [&](bool wait) {
-        while (seen <= lc / 2) {
-            const uint32_t par = (uint32_t)(seen & 1);
-            if (!(wait ? mbar_wait(&sm.ydone, par, a.wait_ns, &sm.abort) : mbar_test(&sm.ydone, par))) return false;
-            ++seen;
-        }
-        const int st = il % kXStages;
-        const uint32_t par = (uint32_t)(((il / kXStages) & 1) ^ 1);
-        if (!(wait ? mbar_wait(&sm.empty[st], par, a.wait_ns, &sm.abort) : mbar_test(&sm.empty[st], par))) return false;
-        mbar_expect_tx(&sm.full[st], kXStage);
-        bulk_g2s(sm.stage[st], Yt + (int64_t)lc * kXChunkA, kXChunkA, &sm.full[st]);
-        bulk_g2s(sm.stage[st] + kXChunkA, a.Lb + ((int64_t)lp * a.nC + lc) * kXChunkB, kXChunkB, &sm.full[st]);
-        ++il;
-        if (++lc == 2 * lp) {
-            lc = 0;
-            ++lp;
-        }
-        return true;
-    };
-    int im = 0;
-    for (int p = 1; p < a.nP && !failed; ++p) {
-        for (int c = 0; c < 2 * p && !failed; ++c, ++im) {
-            if (il == im && !load(true)) {
-                failed = true;
-                break;
-            }
-            while (il < total && il < im + kXStages && load(false)) {
-            }
-            const int set = groups & 1;
+    int im = 0, groups = 0;  // chunks and accumulations issued
+    bool ok = true;
+    for (int p = 1; p < a.nP && ok; ++p)
+        for (int c = 0; c < 2 * p; ++c) {
+            const int set = groups & 1, st = im % kXStages;
             const bool first = c % kXGroup == 0, last = c % kXGroup == kXGroup - 1 || c == 2 * p - 1;
-            if (first && !mbar_wait(&sm.freed[set], (uint32_t)(((groups >> 1) & 1) ^ 1), a.wait_ns, &sm.abort)) {
-                failed = true;
-                break;
-            }
-            const int st = im % kXStages;
-            if (!mbar_wait(&sm.full[st], (uint32_t)((im / kXStages) & 1), a.wait_ns, &sm.abort)) {
-                failed = true;
-                break;
-            }
+            if (first) ok = mbar_wait(&sm.freed[set], (uint32_t)(((groups >> 1) & 1) ^ 1), a.wait_ns, &sm.abort);
+            ok = ok && mbar_wait(&sm.full[st], (uint32_t)((im / kXStages) & 1), a.wait_ns, &sm.abort);
+            if (!ok) break;
             tc_fence_after();
             const uint32_t da = desc_lo(smem_u32(sm.stage[st])), db = desc_lo(smem_u32(sm.stage[st]) + kXChunkA);
             const uint32_t d = tmem + (uint32_t)(set * kXDig * kXB);
@@ -286,18 +281,14 @@ __device__ void issue_all(const XArgs& a, XSmem& sm, const unsigned char* Yt) {
             else
                 mma_chunk<false>(d, da, db);
             mma_commit(&sm.empty[st]);
+            ++im;
             if (last) {
                 mma_commit(&sm.done[set]);
                 ++groups;
             }
         }
-    }
-    if (failed) {
-        atomicExch(&sm.abort, 1);
-        atomicExch(a.timeout, 1);
-    }
-    // copies in flight and the last MMAs, bounded
-    for (int i = im; i < il; ++i) mbar_wait(&sm.full[i % kXStages], (uint32_t)((i / kXStages) & 1), kXWaitNs, nullptr);
+    if (!ok) give_up(a, sm);
+    // the last MMAs, bounded
     if (im > 0)
         mbar_wait(&sm.empty[(im - 1) % kXStages], (uint32_t)(((im - 1) / kXStages) & 1), kXWaitNs, nullptr);
 }
@@ -333,7 +324,9 @@ __global__ void __launch_bounds__(kXThreads, 1) full_fix_tc_kernel(XArgs a) {
     tc_fence_after();
 
     if (warp == 4) {
-        if (lane == 0) issue_all(a, sm, Yt);
+        if (lane == 0) mma_all(a, sm);
+    } else if (warp == 5) {
+        if (lane == 0) copy_all(a, sm, Yt);
     } else {
         const uint64_t K = fix::opaque_mid();
         const int64_t k64 = (int64_t)(blockIdx.x % a.tps) * kXP + tid;
@@ -362,8 +355,7 @@ __global__ void __launch_bounds__(kXThreads, 1) full_fix_tc_kernel(XArgs a) {
                 const int set = groups & 1;
                 if (!failed && !mbar_wait(&sm.done[set], (uint32_t)((groups >> 1) & 1), a.wait_ns, &sm.abort)) {
                     failed = true;
-                    atomicExch(&sm.abort, 1);
-                    atomicExch(a.timeout, 1);
+                    give_up(a, sm);
                 }
                 if (__any_sync(0xffffffffu, failed)) {  // warp-uniform: the loads below are warp-collective
                     failed = true;
