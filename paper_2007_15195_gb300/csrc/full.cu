@@ -108,48 +108,10 @@ __device__ int factor_block(double (*T)[kCholB + 1], const unsigned short* tab, 
     return -1;
 }
 
-// The diagonal block at k0, 512 threads (one trailing entry a thread at the
-// first pivots, so thread 0 holds only the next pivot).  FP64 path: each entry of the factor
-// receives its terms in ascending order with fma and the pivot division last.
-// (Tried for the
-// mixed path and slower: one warp holding the block in registers and
-// shuffling the columns, 49 against 26 us a block, all its FP64 work on one
-// SMSP; the factor repeated by every CTA of the row solve, 70 us a block
-// column, the SMs' FP64 units shared with the trailing update.)
-// upd (mixed path, k0 >= 32): the block first takes the update by the block
-// column before it (rows k0 .. k0 + 31 of that solved panel, fma in ascending
-// column order), which the tensor-core update of that column leaves out, so
-// that this factor waits only for the row solve of the column before and not
-// for the update of its whole first tile column.
-__global__ void __launch_bounds__(512) chol_diag_kernel(double* __restrict__ A, int D, int k0,
-                                                        int* __restrict__ bad, int upd) {
-    __shared__ double T[kCholB][kCholB + 1];
-    __shared__ double P[kCholB][kCholB + 1];
-    __shared__ unsigned short tab[kCholB * (kCholB - 1) / 2];
-    const int b = min(kCholB, D - k0);
-    for (int e = threadIdx.x; e < b * (b + 1) / 2; e += blockDim.x) {
-        int r, c;
-        tri_rc(e, r, c);
-        T[r][c] = A[(int64_t)(k0 + r) * D + k0 + c];
-    }
-    if (upd)
-        for (int x = threadIdx.x; x < b * kCholB; x += blockDim.x) {
-            const int r = x / kCholB, t = x % kCholB;
-            P[r][t] = A[(int64_t)(k0 + r) * D + k0 - kCholB + t];
-        }
-    pair_table(tab);
-    __syncthreads();
-    if (upd) {
-        for (int e = threadIdx.x; e < b * (b + 1) / 2; e += blockDim.x) {
-            int r, c;
-            tri_rc(e, r, c);
-            double acc = T[r][c];
-#pragma unroll
-            for (int t = 0; t < kCholB; ++t) acc = fma(-P[r][t], P[c][t], acc);
-            T[r][c] = acc;
-        }
-        __syncthreads();
-    }
+// Factor the block and store it (all threads); `bad` takes its first
+// non-positive pivot.
+__device__ __forceinline__ void factor_store(double (*T)[kCholB + 1], const unsigned short* tab, int b,
+                                             double* __restrict__ A, int D, int k0, int* __restrict__ bad) {
     const int fail = factor_block(T, tab, b);
     if (fail >= 0) {
         if (threadIdx.x == 0) atomicMin(bad, k0 + fail);
@@ -160,6 +122,77 @@ __global__ void __launch_bounds__(512) chol_diag_kernel(double* __restrict__ A, 
         tri_rc(e, r, c);
         A[(int64_t)(k0 + r) * D + k0 + c] = T[r][c];
     }
+}
+
+// The diagonal block at k0, 512 threads (one trailing entry a thread at the
+// first pivots, so thread 0 holds only the next pivot).  Each entry of the factor
+// receives its terms in ascending order with fma and the pivot division last.
+// (Tried for the
+// mixed path and slower: one warp holding the block in registers and
+// shuffling the columns, 49 against 26 us a block, all its FP64 work on one
+// SMSP; the factor repeated by every CTA of the row solve, 70 us a block
+// column, the SMs' FP64 units shared with the trailing update.)
+__global__ void __launch_bounds__(512) chol_diag_kernel(double* __restrict__ A, int D, int k0,
+                                                        int* __restrict__ bad) {
+    __shared__ double T[kCholB][kCholB + 1];
+    __shared__ unsigned short tab[kCholB * (kCholB - 1) / 2];
+    const int b = min(kCholB, D - k0);
+    for (int e = threadIdx.x; e < b * (b + 1) / 2; e += blockDim.x) {
+        int r, c;
+        tri_rc(e, r, c);
+        T[r][c] = A[(int64_t)(k0 + r) * D + k0 + c];
+    }
+    pair_table(tab);
+    __syncthreads();
+    factor_store(T, tab, b, A, D, k0, bad);
+}
+
+// Mixed path, k0 >= 32: the block first takes the update by the block column
+// before it (rows k0 .. k0 + 31 of that solved panel, fma in ascending column
+// order), which the tensor-core update of that column leaves out, so that this
+// factor waits only for the row solve of the column before and not for the
+// update of its whole first tile column.  The update's 528 x 32 fma hold one SM's
+// FP64 units for 6 us, so a cluster shares them: each CTA takes
+// its part of the entries and leaves them in the first CTA's shared memory, and the
+// first CTA factors the block.
+constexpr int kDiagCluster = 4;  // (2: 7.25 ms a full estimate at D = 2,500; 4 and 8: 7.16; 1: 7.49)
+
+__global__ void __cluster_dims__(kDiagCluster, 1, 1) __launch_bounds__(512)
+    chol_diag_upd_kernel(double* __restrict__ A, int D, int k0, int* __restrict__ bad) {
+    __shared__ double T[kCholB][kCholB + 1];
+    __shared__ double P[kCholB][kCholB + 1];
+    __shared__ unsigned short tab[kCholB * (kCholB - 1) / 2];
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    const int b = min(kCholB, D - k0), n = b * (b + 1) / 2, rank = blockIdx.x;
+    // entry e: e = (warp * kDiagCluster + rank) * 32 + lane, so a rank's warps are its first ones
+    const int e = ((threadIdx.x >> 5) * kDiagCluster + rank) * 32 + (threadIdx.x & 31);
+    int r = 0, c = 0;
+    double acc = 0.0;
+    if (e < n) {
+        tri_rc(e, r, c);
+        acc = A[(int64_t)(k0 + r) * D + k0 + c];
+    }
+    for (int x = threadIdx.x; x < b * kCholB; x += blockDim.x) {
+        const int pr = x / kCholB, t = x % kCholB;
+        P[pr][t] = A[(int64_t)(k0 + pr) * D + k0 - kCholB + t];
+    }
+    if (rank == 0) pair_table(tab);
+    __syncthreads();
+    if (e < n) {
+#pragma unroll
+        for (int t = 0; t < kCholB; ++t) acc = fma(-P[r][t], P[c][t], acc);
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // the first CTA is resident
+    if (e < n) {
+        uint32_t at;
+        asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&T[r][c])));
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(acc) : "memory");
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (rank != 0) return;
+    factor_store(T, tab, b, A, D, k0, bad);
 }
 
 // Rows r >= k0 + 32 of the block column: x L_kk^T = a by forward substitution, one
@@ -362,7 +395,7 @@ struct FullSmem {
 // The contraction's D^2/2 products a point cost 25 cycles a warp instruction
 // triple against the FP64 fma's 76.  (Tiles of 128 points left 152 SMs with 1 or 2
 // tiles each at N S = 24,000.)  D = 1,021, N S = 24,000: 10.6 ms, D = 2,500, N S =
-// 65,536: 134 ms (490 in FP64); the tensor-core form takes 3.8 and 38 ms, so this one serves the
+// 65,536: 134 ms (490 in FP64); the tensor-core form takes 3.5 and 33 ms, so this one serves the
 // smallest problems and histories beyond kFixTcMaxBytes.
 __global__ void __launch_bounds__(kFullThreads) full_genz_kernel(const fix::Digits* __restrict__ Ld,
                                                                  const FixVar* __restrict__ var, FullArgs a,
@@ -554,7 +587,7 @@ cudaError_t enqueue_chol(double* A, int64_t D, int* bad, cudaStream_t st, void* 
     const int64_t nblk = (D + kCholB - 1) / kCholB;
     if (nblk <= 2 || e != cudaSuccess) {  // nothing to overlap
         for (int64_t k0 = 0; k0 < D && e == cudaSuccess; k0 += kCholB) {
-            chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, (int)k0, bad, 0);
+            chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, (int)k0, bad);
             const int64_t rows = D - k0 - kCholB;
             if (rows > 0) {
                 launch_trsm(A, D, k0, st);
@@ -589,7 +622,7 @@ cudaError_t enqueue_chol(double* A, int64_t D, int* bad, cudaStream_t st, void* 
         // k + 1 (which applies column k's update to its own block), then the
         // solve of column k + 1 once the tensor-core update of column k + 1's
         // other rows (side2) is in.  side: the rest of the trailing update.
-        chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, 0, bad, 0);
+        chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, 0, bad);
         for (int64_t k = 0; k < nblk && e == cudaSuccess; ++k) {
             const int64_t k0 = k * kCholB, rows = D - k0 - kCholB;
             if (rows <= 0) break;
@@ -614,7 +647,7 @@ cudaError_t enqueue_chol(double* A, int64_t D, int* bad, cudaStream_t st, void* 
             // block k + 1, which the rest of step k - 1 has updated
             if (k > 0 && e == cudaSuccess) e = cudaStreamWaitEvent(st, ev_rest[(k - 1) & 1], 0);
             if (e == cudaSuccess) {
-                chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, (int)(k0 + kCholB), bad, 1);
+                chol_diag_upd_kernel<<<kDiagCluster, 512, 0, st>>>(A, (int)D, (int)(k0 + kCholB), bad);
                 e = cudaGetLastError();
             }
             if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev_p0[k & 1], 0);
@@ -622,7 +655,7 @@ cudaError_t enqueue_chol(double* A, int64_t D, int* bad, cudaStream_t st, void* 
     }
     for (int64_t k = 0; !tc && k < nblk && e == cudaSuccess; ++k) {
         const int64_t k0 = k * kCholB, rows = D - k0 - kCholB;
-        chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, (int)k0, bad, 0);
+        chol_diag_kernel<<<1, 512, 0, st>>>(A, (int)D, (int)k0, bad);
         if (rows <= 0) {
             e = cudaGetLastError();
             break;
@@ -744,7 +777,7 @@ int64_t full_genz_blocks_per_shift(int64_t N, bool mixed) {
 // Scratch: the shared part (factor, lattice and shift tables, block sums,
 // status words) followed by the precision's own tables and y history.
 // FP64 recursion: the tensor cores' contraction from kFixTcMin variables on (N S =
-// 24,000: D = 64 0.13 against 0.16 ms, D = 256 0.54 against 0.94, D = 1,021 3.8
+// 24,000: D = 64 0.13 against 0.16 ms, D = 256 0.54 against 0.94, D = 1,021 3.5
 // against 10.6), unless its history (16 bytes a y value, twice the integer form's)
 // would not fit beside other work.
 constexpr int64_t kFixTcMin = 64;

@@ -32,8 +32,9 @@
 //
 // Bound by the points' chain of D steps (1.0 us a step) up to D of about 500, then by
 // the history stream (a chunk of 40 KB a us and SM, 5 to 6 TB/s over the GPU; tensor
-// pipe 12 % at D = 640): D = 1,021, N S = 24,000 3.8 ms against 10.6 in integers, D =
-// 2,500, N S = 65,536 38 against 134.
+// pipe 12 % at D = 640): D = 1,021, N S = 24,000 3.5 ms against 10.6 in integers, D =
+// 2,500, N S = 65,536 33 against 134.  (Copies and MMAs from one lane, which refills a
+// stage only after the next chunk's wait: 3.8 and 38 ms.)
 #include <algorithm>
 #include <map>
 #include <mutex>
