@@ -97,11 +97,10 @@ int vecchia_set_stream(vecchia_ctx* ctx, void* cuda_stream);
  * device).  The caller applies perm to sites and u before the next calls.
  * With ctx = NULL both arrays are host memory and the ordering runs on the
  * host (MAXMIN: O(D^2) integer work over the host's cores).  With a context,
- * MAXMIN runs on the device (one persistent CTA: a tournament tree over the
- * distances to the chosen set, each pick scanning only the grid cells within
- * the current maximum distance), with the same result; XY with both arrays
- * on the device and D <= 8192 runs on the device (each site's rank by
- * counting the smaller keys); the other cases run on the host.  MAXMIN: first the site nearest the centre of the quantised
+ * MAXMIN runs on the device (rounds of picks that no open site in reach
+ * dominates, then a sort of their keys), with the same result; XY with both
+ * arrays on the device runs there (a merge sort; on the host where its scratch
+ * does not fit); the other cases run on the host.  MAXMIN: first the site nearest the centre of the quantised
  * bounding box, then repeatedly the site farthest from the chosen ones, on
  * quantised coordinates, ties to the smaller index. */
 int vecchia_order(vecchia_ctx* ctx, const double* sites, int64_t D, int kind, int32_t* perm);
@@ -142,9 +141,8 @@ int vecchia_log_cdf_terms(vecchia_ctx* ctx, const double* sites_ordered, int64_t
 
 /* Steps a0-a7 in one call from unordered sites: the ordering (order_kind),
  * its application, the m-neighbour rows and the log-CDF, queued on the
- * context's stream with no host round trip in between (the XY ordering of
- * more than 8192 sites is the one host step); the same results as the four
- * calls in sequence.  sites (D x 2) and u (D) host or device, both of one
+ * context's stream with no host round trip in between; the same results as
+ * the four calls in sequence.  sites (D x 2) and u (D) host or device, both of one
  * kind; perm_out (D, host or device) may be NULL, else it gets the ordering
  * (new position -> old index).  Other arguments as for vecchia_log_cdf. */
 int vecchia_log_cdf_unordered(vecchia_ctx* ctx, const double* sites, const double* u, int64_t D, int order_kind,
@@ -321,10 +319,12 @@ int vecchia_mixture_log_cdf(vecchia_ctx* ctx, const double* sites_ordered, int64
  * the FP32 operands -- FP32-level accuracy --, FP64 running product and
  * sums).  log_p = log of the mean over shifts of the lattice means; rel_se =
  * their standard error over the mean.  Arrays host or device (both of one
- * kind); device memory grows as about 16 D^2 + 9.2 (mixed) or 8 (FP64) D S N
- * bytes.  D <= VECCHIA_FULL_MAX_D.  A non-positive pivot gives
+ * kind); device memory grows as about 16 D^2 + 9.2 (mixed) or 16 (FP64: its
+ * conditional means on the tensor cores too, exact sums of 64-bit fixed-point
+ * products; 8 beyond 96 GB or where 16 does not fit, in integer products)
+ * D S N bytes.  D <= VECCHIA_FULL_MAX_D.  A non-positive pivot gives
  * VECCHIA_ERR_NOT_PD with its site in vecchia_last_error_site();
- * VECCHIA_ERR_TIMEOUT means a bounded device wait of the mixed recursion ran
+ * VECCHIA_ERR_TIMEOUT means a bounded device wait of a tensor-core kernel ran
  * out (2 s without progress). */
 #define VECCHIA_FULL_MAX_D 32768
 int vecchia_full_genz(vecchia_ctx* ctx, const double* sites_ordered, int64_t D, vecchia_cov cov,

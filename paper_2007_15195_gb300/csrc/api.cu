@@ -956,10 +956,11 @@ int vecchia_order(vecchia_ctx* c, const double* sites, int64_t D, int kind, int3
     // with no context both arrays are host memory and the ordering runs on the host
     const bool dev_in = c && is_device_ptr(sites), dev_out = c && is_device_ptr(perm);
     if (c && (dev_in || dev_out) && cudaSetDevice(c->device) != cudaSuccess) return VECCHIA_ERR_CUDA;
-    if (c && kind == VECCHIA_ORDER_XY && dev_in && dev_out) {
-        // XY on the device
-        int st = ensure_arena(c, vk::order_xy_scratch_bytes(D));
-        if (st != VECCHIA_OK) return st;
+    // the device orderings index 2 D entries in 32 bits; beyond, the host's
+    const bool dev_sized = c && D <= INT_MAX / 2;
+    // XY on the device, or on the host where its scratch does not fit
+    if (dev_sized && kind == VECCHIA_ORDER_XY && dev_in && dev_out &&
+        ensure_arena(c, vk::order_xy_scratch_bytes(D)) == VECCHIA_OK) {
         const cudaError_t e = vk::launch_order_xy(sites, D, perm, c->arena, c->stream);
         if (e != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess) {
             cudaGetLastError();
@@ -967,7 +968,7 @@ int vecchia_order(vecchia_ctx* c, const double* sites, int64_t D, int kind, int3
         }
         return VECCHIA_OK;
     }
-    if (c && kind == VECCHIA_ORDER_MAXMIN) {  // exact maxmin on the device
+    if (dev_sized && kind == VECCHIA_ORDER_MAXMIN) {  // exact maxmin on the device
         if (cudaSetDevice(c->device) != cudaSuccess) return VECCHIA_ERR_CUDA;
         Carve dv(nullptr);
         const size_t o_s = dv.off;
@@ -1374,8 +1375,12 @@ int vecchia_full_genz(vecchia_ctx* c, const double* sites, int64_t D, vecchia_co
     const size_t o_u = dv.off;
     if (!dev_in) dv.take<double>(D);
     const size_t o_scr = dv.off;
-    dv.take<char>(vk::full_genz_scratch_bytes(D, N, S, mixed));
-    int st = ensure_arena(c, dv.off);
+    bool tc64 = !mixed && vk::full_fix_tc_pays(D, N, S);
+    int st = ensure_arena(c, o_scr + vk::full_genz_scratch_bytes(D, N, S, mixed, tc64));
+    if (st == VECCHIA_ERR_NOMEM && tc64) {  // the integer form keeps half the history
+        tc64 = false;
+        st = ensure_arena(c, o_scr + vk::full_genz_scratch_bytes(D, N, S, mixed, tc64));
+    }
     if (st != VECCHIA_OK) return st;
     char* A = (char*)c->arena;
     const double* sd = dev_in ? sites : (const double*)(A + o_s);
@@ -1388,7 +1393,7 @@ int vecchia_full_genz(vecchia_ctx* c, const double* sites, int64_t D, vecchia_co
     if (e == cudaSuccess && !dev_in)
         e = cudaMemcpyAsync(A + o_u, u, sizeof(double) * D, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
-        e = vk::launch_full_genz(sd, ud, D, cov, N, S, mixed, g.data(), gfix.data(), seed, A + o_scr, part.data(),
+        e = vk::launch_full_genz(sd, ud, D, cov, N, S, mixed, tc64, g.data(), gfix.data(), seed, A + o_scr, part.data(),
                                  &bad, &timed_out, c->full_wait_ns, c->full_withhold,
                                  c->timing ? c->ev0 : nullptr, c->timing ? c->ev1 : nullptr, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

@@ -779,14 +779,15 @@ int64_t full_genz_blocks_per_shift(int64_t N, bool mixed) {
 // FP64 recursion: the tensor cores' contraction from kFixTcMin variables on (N S =
 // 24,000: D = 64 0.13 against 0.16 ms, D = 256 0.54 against 0.94, D = 1,021 3.5
 // against 10.6), unless its history (16 bytes a y value, twice the integer form's)
-// would not fit beside other work.
+// would crowd out other work; the caller takes the integer form, too, where this
+// one's scratch cannot be allocated.
 constexpr int64_t kFixTcMin = 64;
 constexpr size_t kFixTcMaxBytes = 96ull << 30;
-bool fix_tc_pays(int64_t D, int64_t N, int S) {
+bool full_fix_tc_pays(int64_t D, int64_t N, int S) {
     return D >= kFixTcMin && full_fix_tc_scratch_bytes(D, N, S) <= kFixTcMaxBytes;
 }
 
-size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed) {
+size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed, bool tc64) {
     const int64_t bps = (N + kFullP - 1) / kFullP, nblk = full_genz_blocks_per_shift(N, mixed);
     const int64_t dim = D > 1 ? D - 1 : 1;
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
@@ -794,13 +795,13 @@ size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed) {
                           al(sizeof(uint32_t) * S * dim) + al(sizeof(double) * S * nblk) + al(2 * sizeof(int)) +
                           al(sizeof(uint64_t) + 2 * sizeof(int64_t) + sizeof(int32_t));
     if (mixed) return shared + al(chol_tc_scratch_bytes(D)) + full_tc_scratch_bytes(D, N, S);
-    if (fix_tc_pays(D, N, S)) return shared + full_fix_tc_scratch_bytes(D, N, S);
+    if (tc64) return shared + full_fix_tc_scratch_bytes(D, N, S);
     return shared + al(sizeof(fix::Digits) * D * D) + al(sizeof(FixVar) * D) +
            al(sizeof(fix::Digits) * (size_t)S * bps * D * kFullP);
 }
 
 cudaError_t launch_full_genz(const double* sites, const double* u, int64_t D, const vecchia_cov& cov, int64_t N,
-                             int S, bool mixed, const uint32_t* g_host, const uint32_t* gfix_host,
+                             int S, bool mixed, bool tc64, const uint32_t* g_host, const uint32_t* gfix_host,
                              uint64_t seed, void* scratch, double* part_host, int* bad_host, int* timeout_host,
                              uint64_t wait_ns, int withhold, cudaEvent_t ev_begin, cudaEvent_t ev_end,
                              cudaStream_t st) {
@@ -848,7 +849,7 @@ cudaError_t launch_full_genz(const double* sites, const double* u, int64_t D, co
     if (mixed) {
         e = launch_full_genz_tc(A, u, D, N, S, gdev + dim, dfix, (int)dim, p, part, bad + 1, wait_ns, withhold,
                                 ev_begin, ev_end, st);
-    } else if (fix_tc_pays(D, N, S)) {
+    } else if (tc64) {
         e = cudaMemsetAsync(part, 0, sizeof(double) * S * nblk, st);
         if (e == cudaSuccess)
             e = launch_full_fix_tc(A, u, D, N, S, gdev, delta, (int)dim, p, part, (int)nblk, bad + 1, wait_ns, ev_begin,

@@ -1,9 +1,9 @@
 // genz.cu -- the fused per-term kernel of the Vecchia log-CDF and the log-sum.
 //
 // One CTA takes one Vecchia term at a time (a site i of a problem):
-//   prologue (one warp, FP64): the block b = (N_i ascending, i) of
+//   prologue (FP64, all warps): the block b = (N_i ascending, i) of
 //     Sec. 2.2 / Eq. (vecchia-cdf), its covariance from the covariance
-//     function (Sec. 3, Sec. 4.1), the Cholesky factor with lanes over rows;
+//     function (Sec. 3, Sec. 4.1), the Cholesky factor;
 //   body (all warps): Genz's separation-of-variables recursion at the
 //     shifted lattice points, one lane per point, the numerator (d-dim) and
 //     denominator ((d-1)-dim, the leading block) sharing every sample;

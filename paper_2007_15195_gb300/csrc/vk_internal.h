@@ -182,7 +182,9 @@ cudaError_t launch_conditioning(const double* L, int k, const double* sites_i, c
 // Full D-dimensional Genz estimate (full.cu): covariance, blocked FP64
 // Cholesky, Genz over all variables; part_host gets S x ceil(N/128) tile sums
 // of the point products, *bad_host the first non-positive pivot (INT_MAX if none).
-size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed);
+// tc64: the FP64 recursion's contraction on the tensor cores (full_fix_tc_pays: worth it).
+bool full_fix_tc_pays(int64_t D, int64_t N, int S);
+size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed, bool tc64);
 // Point-block sums per shift written by launch_full_genz.
 int64_t full_genz_blocks_per_shift(int64_t N, bool mixed);
 // part_host: per-shift point-block sums (S x full_genz_blocks_per_shift); bad_host:
@@ -190,7 +192,7 @@ int64_t full_genz_blocks_per_shift(int64_t N, bool mixed);
 // wait of the tensor-core kernel ran out; ev_begin / ev_end (may be null) are
 // recorded around the recursion kernel alone.
 cudaError_t launch_full_genz(const double* sites, const double* u, int64_t D, const vecchia_cov& cov, int64_t N,
-                             int S, bool mixed, const uint32_t* g_host, const uint32_t* gfix_host,
+                             int S, bool mixed, bool tc64, const uint32_t* g_host, const uint32_t* gfix_host,
                              uint64_t seed, void* scratch, double* part_host, int* bad_host, int* timeout_host,
                              uint64_t wait_ns, int withhold, cudaEvent_t ev_begin, cudaEvent_t ev_end,
                              cudaStream_t st);

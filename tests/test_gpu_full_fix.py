@@ -48,3 +48,24 @@ def test_threshold_ranges(ctx, D, deep):
     u[3::deep] = -7.5
     u[5::41] = 1e300
     _check(ctx, s, (1, 1.0, 0.15, 1.5, 0.0), u, 140, 4, 9)
+
+
+def test_scratch_limit(ctx):
+    """With room for the integer form's history (3.4 GB) but not for the tensor-core
+    form's (7.5 GB), the call takes the integer form."""
+    import torch
+    D, N, S = 200, 1 << 19, 4
+    s = inputs.uniform_sites(D, 77)
+    u = inputs.rng(D, 1).normal(0.6, 0.4, size=D)
+    cov = (0, 1.0, 0.2, 0.5, 0.0)
+    c = B.Context(0)
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (5 << 30), dtype=torch.uint8, device="cuda")
+    try:
+        few = B.vecchia_full_genz(c, s, cov, u, N, S, 5, B.FP64)
+    finally:
+        c.close()
+        del hold
+        torch.cuda.empty_cache()
+    full = B.vecchia_full_genz(ctx, s, cov, u, N, S, 5, B.FP64)
+    assert abs(few[0] - full[0]) <= 1e-10 * max(1.0, abs(full[0]))
+    assert abs(few[1] - full[1]) <= 1e-8 * full[1]
