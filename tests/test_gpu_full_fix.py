@@ -51,15 +51,15 @@ def test_threshold_ranges(ctx, D, deep):
 
 
 def test_scratch_limit(ctx):
-    """With room for the integer form's history (3.4 GB) but not for the tensor-core
-    form's (7.5 GB), the call takes the integer form."""
+    """With room for the integer form's history (2.1 GB) but not for the tensor-core
+    form's (4.3 GB), the call takes the integer form."""
     import torch
-    D, N, S = 200, 1 << 19, 4
+    D, N, S = 1024, 4096, 64
     s = inputs.uniform_sites(D, 77)
     u = inputs.rng(D, 1).normal(0.6, 0.4, size=D)
     cov = (0, 1.0, 0.2, 0.5, 0.0)
     c = B.Context(0)
-    hold = torch.empty(torch.cuda.mem_get_info()[0] - (5 << 30), dtype=torch.uint8, device="cuda")
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (13 << 28), dtype=torch.uint8, device="cuda")
     try:
         few = B.vecchia_full_genz(c, s, cov, u, N, S, 5, B.FP64)
     finally:
