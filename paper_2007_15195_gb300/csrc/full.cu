@@ -395,7 +395,7 @@ struct FullSmem {
 // The contraction's D^2/2 products a point cost 25 cycles a warp instruction
 // triple against the FP64 fma's 76.  (Tiles of 128 points left 152 SMs with 1 or 2
 // tiles each at N S = 24,000.)  D = 1,021, N S = 24,000: 10.6 ms, D = 2,500, N S =
-// 65,536: 134 ms (490 in FP64); the tensor-core form takes 3.5 and 33 ms, so this one serves the
+// 65,536: 134 ms (490 in FP64); the tensor-core form takes 3.1 and 31 ms, so this one serves the
 // smallest problems and histories beyond kFixTcMaxBytes.
 __global__ void __launch_bounds__(kFullThreads) full_genz_kernel(const fix::Digits* __restrict__ Ld,
                                                                  const FixVar* __restrict__ var, FullArgs a,
@@ -777,7 +777,7 @@ int64_t full_genz_blocks_per_shift(int64_t N, bool mixed) {
 // Scratch: the shared part (factor, lattice and shift tables, block sums,
 // status words) followed by the precision's own tables and y history.
 // FP64 recursion: the tensor cores' contraction from kFixTcMin variables on (N S =
-// 24,000: D = 64 0.13 against 0.16 ms, D = 256 0.54 against 0.94, D = 1,021 3.5
+// 24,000: D = 64 0.08 against 0.16 ms, D = 256 0.39 against 0.94, D = 1,021 3.1
 // against 10.6), unless its history (16 bytes a y value, twice the integer form's)
 // would crowd out other work; the caller takes the integer form, too, where this
 // one's scratch cannot be allocated.

@@ -16,15 +16,17 @@
 // integer form's own rounding (below 2 units a product, 0.2 rms, at 2^-60 of the
 // row's largest possible sum).
 //
-// A CTA takes 128 lattice points (MMA rows).  Four warps, one thread a point, run the
-// panels: they add the accumulators of each group of 128 variables to the points'
+// A CTA takes one or two tiles of 128 lattice points (MMA rows).  Four warps a tile, one
+// thread a point, run the panels: they add the accumulators of each group of 128 variables to the points'
 // sums in shared memory, run the panel's variables in order, and write their y
-// as digits to the history.  One lane of a fifth warp streams history chunks of 16
+// as digits to the history.  One lane of another warp streams history chunks of 16
 // variables (32 KB of y digits, 8 KB of the panel's L digits) with cp.async.bulk
-// through a three-stage ring; one lane of a sixth issues 36 MMAs (M = 128, N = 32, K = 16)
-// a chunk.  Two sets of accumulators (2 x 8 x 32 columns) alternate between groups, so they
-// run up to two groups ahead, into the next panel during the points' pass; only
-// the chunks of that pass wait for it.  Operands lie in no-swizzle K-major core matrices
+// through a ring of three stages (two tiles: two); one lane of a further one issues 36 MMAs
+// (M = 128, N = 32, K = 16) a chunk.  There are two sets of accumulators (2 x 8 x 32 columns).  With one
+// tile they alternate between groups, so the MMAs run up to two groups ahead, into the next
+// panel during the points' pass; only the chunks of that pass wait for it.  Two tiles
+// have one set each: one's MMAs run beside the other's additions, and the passes' chains,
+// twice the warps an SMSP, hide each other's latency.  Operands lie in no-swizzle K-major core matrices
 // (8 rows x 16 bytes): per group of 8 rows the eight digit matrices of a chunk,
 // 256 bytes each (K stride 128 bytes, row-group stride 2,048).  Every wait is bounded by
 // the global timer; on expiry the kernel records a timeout, waits (bounded) for
@@ -32,9 +34,9 @@
 //
 // Bound by the points' chain of D steps (1.0 us a step) up to D of about 500, then by
 // the history stream (a chunk of 40 KB a us and SM, 5 to 6 TB/s over the GPU; tensor
-// pipe 12 % at D = 640): D = 1,021, N S = 24,000 3.5 ms against 10.6 in integers, D =
-// 2,500, N S = 65,536 33 against 134.  (Copies and MMAs from one lane, which refills a
-// stage only after the next chunk's wait: 3.8 and 38 ms.)
+// pipe 12 % at D = 640): D = 1,021, N S = 24,000 3.1 ms against 10.6 in integers, D =
+// 2,500, N S = 65,536 31 against 134.  (One tile a CTA: 3.5 and 33; with copies and MMAs
+// from one lane, which refills a stage only after the next chunk's wait: 3.8 and 38 ms.)
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -45,13 +47,17 @@
 namespace vk {
 namespace {
 
-constexpr int kXP = 128;       // lattice points per CTA = MMA M
+constexpr int kXP = 128;       // lattice points per tile = MMA M
 constexpr int kXB = 32;        // panel width = MMA N
 constexpr int kXK = 16;        // history chunk (variables) = MMA K
 constexpr int kXDig = 8;       // digits
 constexpr int kXGroup = 8;     // chunks per accumulation
-constexpr int kXStages = 3;
-constexpr int kXThreads = kXP + 64;  // point warps, the MMA warp, the copy warp
+// H halves of 128 points a CTA (1 or 2): stages of the ring, threads (point warps, the MMA
+// warp, the copy warp)
+template <int H>
+constexpr int kXStages = H == 1 ? 3 : 2;
+template <int H>
+constexpr int kXThreads = H * kXP + 64;
 constexpr uint32_t kRowGroup = kXDig * 256;               // 8 rows: eight 256-byte digit matrices
 constexpr uint32_t kXChunkA = (kXP / 8) * kRowGroup;      // 32,768
 constexpr uint32_t kXChunkB = (kXB / 8) * kRowGroup;      // 8,192
@@ -63,23 +69,25 @@ constexpr uint64_t kXWaitNs = 2000000000ull;
 constexpr uint32_t kXIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kXB >> 3) << 17) |
                              ((uint32_t)(kXP >> 4) << 24);
 
+template <int H>
 struct XSmem {
-    __align__(1024) unsigned char stage[kXStages][kXStage];
+    __align__(1024) unsigned char stage[kXStages<H>][kXStage];
     fix::FixTables tb;
-    __align__(16) int64_t Z[kXB][kXP];                  // conditional sums, then the panel's y (digits)
+    __align__(16) int64_t Z[kXB][H * kXP];                // conditional sums, then the panel's y (digits)
     __align__(16) fix::Digits Lp[kXB][kXB + 1];         // the panel's own triangle
     FixVar var[kXB];
     uint64_t G[kXB], Dt[kXB];                           // lattice multipliers and this shift, 64-bit fixed point
-    double red[kXP / 32];
-    __align__(8) uint64_t full[kXStages], empty[kXStages], done[2], freed[2], ydone;
+    double red[H * kXP / 32];
+    __align__(8) uint64_t full[kXStages<H>], empty[kXStages<H>], done[2], freed[2], ydone[H];
     uint32_t tmem;
     int abort, nan;
 };
+static_assert(sizeof(XSmem<1>) <= 227 * 1024 && sizeof(XSmem<2>) <= 227 * 1024, "one CTA's shared memory");
 
 struct XArgs {
     int D, nP, nC;              // variables, panels, chunks of 16
     int64_t N;
-    int tps;                    // tiles per shift
+    int tps;                    // CTAs per shift
     const uint32_t* g;          // lattice vector, D - 1 entries
     const double* delta;        // S x dim shifts
     const double* u;            // thresholds (for NaN only: its result is NaN)
@@ -88,7 +96,7 @@ struct XArgs {
     const unsigned char* Lb;    // digits of -L, [nP][nC] blocks of 8 KB (columns before the panel)
     const fix::Digits* Lp;      // [nP][32][32]: the panel's own triangle of -L
     unsigned char* Y;           // history digits, [tiles][nC] chunks of 32 KB
-    double* part;               // per shift part_stride sums, the first tps of them ours
+    double* part;               // per shift part_stride sums, the first H tps of them ours
     int part_stride;
     int* timeout;
     uint64_t wait_ns;
@@ -180,7 +188,10 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void points_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+template <int H>
+__device__ __forceinline__ void points_sync() {
+    asm volatile("bar.sync 1, %0;" ::"n"(H * kXP) : "memory");
+}
 
 // The eight balanced base-256 digits of X (top digit last to leave: within +-128), as bf16 bits.
 __device__ __forceinline__ void digit_bits(int64_t X, uint32_t (&d)[kXDig]) {
@@ -231,83 +242,101 @@ __global__ void __launch_bounds__(128) fix_tc_tables_kernel(const double* __rest
             (v < D && v0 + tid < v) ? fix_coef(row[v0 + tid], kL) : fix::Digits{0, 0};
 }
 
-__device__ void give_up(const XArgs& a, XSmem& sm) {
+template <int H>
+__device__ void give_up(const XArgs& a, XSmem<H>& sm) {
     atomicExch(&sm.abort, 1);
     atomicExch(a.timeout, 1);
 }
 
+// Accumulation n of a half (its groups counted over all panels): the accumulator set,
+// and how often that set was used before.  One half alternates between the two sets, two
+// halves have one each.
+template <int H>
+__device__ __forceinline__ int acc_set(int n, int h) { return H == 1 ? n & 1 : h; }
+template <int H>
+__device__ __forceinline__ uint32_t acc_use(int n) { return (uint32_t)(H == 1 ? n >> 1 : n); }
+
 // The copies of every panel, by one lane of its own (a lane that also issued the
 // MMAs refilled a stage only after the next chunk's wait): chunk c < 2 p of panel p
 // once the points have written the panel that it holds and its stage is free.
-__device__ void copy_all(const XArgs& a, XSmem& sm, const unsigned char* Yt) {
-    int il = 0, seen = 0;  // copies issued; panels whose y the points have written
+template <int H>
+__device__ void copy_all(const XArgs& a, XSmem<H>& sm, const unsigned char* Yt) {
+    constexpr int ST = kXStages<H>;
+    int il = 0, seen[H] = {};  // copies issued; panels whose y a half's points have written
     bool ok = true;
     for (int p = 1; p < a.nP && ok; ++p)
-        for (int c = 0; c < 2 * p && ok; ++c) {
-            while (ok && seen <= c / 2) {
-                ok = mbar_wait(&sm.ydone, (uint32_t)(seen & 1), a.wait_ns, &sm.abort);
-                ++seen;
-            }
-            const int st = il % kXStages;
-            ok = ok && mbar_wait(&sm.empty[st], (uint32_t)(((il / kXStages) & 1) ^ 1), a.wait_ns, &sm.abort);
-            if (!ok) break;
-            mbar_expect_tx(&sm.full[st], kXStage);
-            bulk_g2s(sm.stage[st], Yt + (int64_t)c * kXChunkA, kXChunkA, &sm.full[st]);
-            bulk_g2s(sm.stage[st] + kXChunkA, a.Lb + ((int64_t)p * a.nC + c) * kXChunkB, kXChunkB, &sm.full[st]);
-            ++il;
-        }
+        for (int c0 = 0; c0 < 2 * p && ok; c0 += kXGroup)
+#pragma unroll
+            for (int h = 0; h < H; ++h)
+                for (int c = c0; c < min(c0 + kXGroup, 2 * p) && ok; ++c) {
+                    while (ok && seen[h] <= c / 2) {
+                        ok = mbar_wait(&sm.ydone[h], (uint32_t)(seen[h] & 1), a.wait_ns, &sm.abort);
+                        ++seen[h];
+                    }
+                    const int st = il % ST;
+                    ok = ok && mbar_wait(&sm.empty[st], (uint32_t)(((il / ST) & 1) ^ 1), a.wait_ns, &sm.abort);
+                    if (!ok) break;
+                    mbar_expect_tx(&sm.full[st], kXStage);
+                    bulk_g2s(sm.stage[st], Yt + ((int64_t)h * a.nC + c) * kXChunkA, kXChunkA, &sm.full[st]);
+                    bulk_g2s(sm.stage[st] + kXChunkA, a.Lb + ((int64_t)p * a.nC + c) * kXChunkB, kXChunkB, &sm.full[st]);
+                    ++il;
+                }
     if (!ok) give_up(a, sm);
     // the copies in flight, bounded
-    for (int i = max(0, il - kXStages); i < il; ++i)
-        mbar_wait(&sm.full[i % kXStages], (uint32_t)((i / kXStages) & 1), kXWaitNs, nullptr);
+    for (int i = max(0, il - ST); i < il; ++i)
+        mbar_wait(&sm.full[i % ST], (uint32_t)((i / ST) & 1), kXWaitNs, nullptr);
 }
 
-// The MMAs of every panel, by one lane.
-__device__ void mma_all(const XArgs& a, XSmem& sm) {
+// The MMAs of every panel, by one lane, in the copies' order: a group of one half, then
+// the same of the other, so that one's MMAs run beside the other's additions.
+template <int H>
+__device__ void mma_all(const XArgs& a, XSmem<H>& sm) {
+    constexpr int ST = kXStages<H>;
     const uint32_t tmem = sm.tmem;
-    int im = 0, groups = 0;  // chunks and accumulations issued
+    int im = 0, n = 0;  // chunks issued; accumulations of a half
     bool ok = true;
     for (int p = 1; p < a.nP && ok; ++p)
-        for (int c = 0; c < 2 * p; ++c) {
-            const int set = groups & 1, st = im % kXStages;
-            const bool first = c % kXGroup == 0, last = c % kXGroup == kXGroup - 1 || c == 2 * p - 1;
-            if (first) ok = mbar_wait(&sm.freed[set], (uint32_t)(((groups >> 1) & 1) ^ 1), a.wait_ns, &sm.abort);
-            ok = ok && mbar_wait(&sm.full[st], (uint32_t)((im / kXStages) & 1), a.wait_ns, &sm.abort);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t da = desc_lo(smem_u32(sm.stage[st])), db = desc_lo(smem_u32(sm.stage[st]) + kXChunkA);
-            const uint32_t d = tmem + (uint32_t)(set * kXDig * kXB);
-            if (first)
-                mma_chunk<true>(d, da, db);
-            else
-                mma_chunk<false>(d, da, db);
-            mma_commit(&sm.empty[st]);
-            ++im;
-            if (last) {
-                mma_commit(&sm.done[set]);
-                ++groups;
+        for (int c0 = 0; c0 < 2 * p && ok; c0 += kXGroup, ++n)
+            for (int h = 0; h < H && ok; ++h) {
+                const int set = acc_set<H>(n, h);
+                const uint32_t d = tmem + (uint32_t)(set * kXDig * kXB);
+                ok = mbar_wait(&sm.freed[set], (acc_use<H>(n) & 1) ^ 1, a.wait_ns, &sm.abort);
+                for (int c = c0; c < min(c0 + kXGroup, 2 * p); ++c) {
+                    const int st = im % ST;
+                    ok = ok && mbar_wait(&sm.full[st], (uint32_t)((im / ST) & 1), a.wait_ns, &sm.abort);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t da = desc_lo(smem_u32(sm.stage[st])), db = desc_lo(smem_u32(sm.stage[st]) + kXChunkA);
+                    if (c == c0)
+                        mma_chunk<true>(d, da, db);
+                    else
+                        mma_chunk<false>(d, da, db);
+                    mma_commit(&sm.empty[st]);
+                    ++im;
+                }
+                if (ok) mma_commit(&sm.done[set]);
             }
-        }
     if (!ok) give_up(a, sm);
     // the last MMAs, bounded
-    if (im > 0)
-        mbar_wait(&sm.empty[(im - 1) % kXStages], (uint32_t)(((im - 1) / kXStages) & 1), kXWaitNs, nullptr);
+    if (im > 0) mbar_wait(&sm.empty[(im - 1) % ST], (uint32_t)(((im - 1) / ST) & 1), kXWaitNs, nullptr);
 }
 
-__global__ void __launch_bounds__(kXThreads, 1) full_fix_tc_kernel(XArgs a) {
+template <int H>
+__global__ void __launch_bounds__(kXThreads<H>, 1) full_fix_tc_kernel(XArgs a) {
     extern __shared__ __align__(1024) unsigned char x_smem[];
-    XSmem& sm = *reinterpret_cast<XSmem*>(x_smem);
+    XSmem<H>& sm = *reinterpret_cast<XSmem<H>*>(x_smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, D = a.D;
     const int s = blockIdx.x / a.tps;
-    unsigned char* Yt = a.Y + (int64_t)blockIdx.x * a.nC * kXChunkA;
-    if (warp == 4) {
+    constexpr int kMmaWarp = H * kXP / 32, kCopyWarp = kMmaWarp + 1;
+    unsigned char* Yt = a.Y + (int64_t)blockIdx.x * H * a.nC * kXChunkA;  // its halves' histories
+    if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem)),
                      "r"(kXCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int i = 0; i < kXStages; ++i) {
+        for (int i = 0; i < kXStages<H>; ++i) {
             mbar_init(&sm.full[i], 1);
             mbar_init(&sm.empty[i], 1);
         }
@@ -315,7 +344,7 @@ __global__ void __launch_bounds__(kXThreads, 1) full_fix_tc_kernel(XArgs a) {
             mbar_init(&sm.done[i], 1);
             mbar_init(&sm.freed[i], kXP);
         }
-        mbar_init(&sm.ydone, kXP);
+        for (int h = 0; h < H; ++h) mbar_init(&sm.ydone[h], kXP);
         sm.abort = sm.nan = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -324,22 +353,23 @@ __global__ void __launch_bounds__(kXThreads, 1) full_fix_tc_kernel(XArgs a) {
     __syncthreads();
     tc_fence_after();
 
-    if (warp == 4) {
+    if (warp == kMmaWarp) {
         if (lane == 0) mma_all(a, sm);
-    } else if (warp == 5) {
+    } else if (warp == kCopyWarp) {
         if (lane == 0) copy_all(a, sm, Yt);
     } else {
         const uint64_t K = fix::opaque_mid();
-        const int64_t k64 = (int64_t)(blockIdx.x % a.tps) * kXP + tid;
+        const int64_t k64 = (int64_t)(blockIdx.x % a.tps) * (H * kXP) + tid;
+        const int h = tid / kXP, row = tid % kXP;
         const bool valid = k64 < a.N;
         const uint32_t k = (uint32_t)(valid ? k64 : a.N - 1);
-        const uint32_t trow = sm.tmem + ((uint32_t)(warp * 32) << 16);
+        const uint32_t trow = sm.tmem + ((uint32_t)((warp & 3) * 32) << 16);
         fix::FixFloat f{~0ull, 0};
         int groups = 0;
         bool failed = false;
         for (int p = 0; p < a.nP; ++p) {
             const int v0 = p * kXB, nb = min(kXB, D - v0);
-            points_sync();  // the last panel's constants are no longer read
+            points_sync<H>();  // the last panel's constants are no longer read
             if (tid < nb) {
                 const int v = v0 + tid;
                 sm.var[tid] = a.var[v];
@@ -347,14 +377,14 @@ __global__ void __launch_bounds__(kXThreads, 1) full_fix_tc_kernel(XArgs a) {
                 sm.G[tid] = v < D - 1 ? fix64_ratio(a.g[v], (uint64_t)a.N) : 0;
                 sm.Dt[tid] = v < D - 1 ? fix_shift(a.delta[(int64_t)s * a.dim + v]) : 0;
             }
-            for (int x = tid; x < kXB * kXB; x += kXP) sm.Lp[x / kXB][x % kXB] = a.Lp[(int64_t)p * kXB * kXB + x];
-            points_sync();
+            for (int x = tid; x < kXB * kXB; x += H * kXP) sm.Lp[x / kXB][x % kXB] = a.Lp[(int64_t)p * kXB * kXB + x];
+            points_sync<H>();
             for (int j = 0; j < nb; ++j) sm.Z[j][tid] = sm.var[j].up;
             // add the accumulators, 128 variables of the history at a time
             const int n_groups = (2 * p + kXGroup - 1) / kXGroup;
             for (int gi = 0; gi < n_groups; ++gi, ++groups) {
-                const int set = groups & 1;
-                if (!failed && !mbar_wait(&sm.done[set], (uint32_t)((groups >> 1) & 1), a.wait_ns, &sm.abort)) {
+                const int set = acc_set<H>(groups, h);
+                if (!failed && !mbar_wait(&sm.done[set], acc_use<H>(groups) & 1, a.wait_ns, &sm.abort)) {
                     failed = true;
                     give_up(a, sm);
                 }
@@ -407,7 +437,8 @@ __global__ void __launch_bounds__(kXThreads, 1) full_fix_tc_kernel(XArgs a) {
                         fix_quantile(sm.tb, (uint64_t)k * sm.G[j] + sm.Dt[j], e, K);
             }
             if (p + 1 < a.nP) {  // a full panel: its y as digits, eight variables (16 bytes a digit) at a time
-                unsigned char* dst = Yt + (int64_t)(2 * p) * kXChunkA + (tid / 8) * kRowGroup + (tid % 8) * 16;
+                unsigned char* dst =
+                    Yt + ((int64_t)h * a.nC + 2 * p) * kXChunkA + (row / 8) * kRowGroup + (row % 8) * 16;
 #pragma unroll 1
                 for (int o = 0; o < kXB / 8; ++o) {
                     uint32_t w[kXDig][4];
@@ -427,7 +458,7 @@ __global__ void __launch_bounds__(kXThreads, 1) full_fix_tc_kernel(XArgs a) {
                         *reinterpret_cast<uint4*>(at + i * 256) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
                 }
                 asm volatile("fence.proxy.async.global;" ::: "memory");
-                mbar_arrive(&sm.ydone);
+                mbar_arrive(&sm.ydone[h]);
             }
         }
         // tile sum of the point products, fixed order
@@ -435,18 +466,54 @@ __global__ void __launch_bounds__(kXThreads, 1) full_fix_tc_kernel(XArgs a) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) sm.red[warp] = v;
-        points_sync();
-        if (tid == 0) {
+        points_sync<H>();
+        if (row == 0) {
             double t = 0.0;
-            for (int w = 0; w < kXP / 32; ++w) t += sm.red[w];
-            a.part[(int64_t)s * a.part_stride + blockIdx.x % a.tps] = sm.nan ? __longlong_as_double(0x7ff8000000000000LL) : t;
+            for (int w = 0; w < kXP / 32; ++w) t += sm.red[h * (kXP / 32) + w];
+            a.part[(int64_t)s * a.part_stride + (blockIdx.x % a.tps) * H + h] = sm.nan ? __longlong_as_double(0x7ff8000000000000LL) : t;
         }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 4)
+    if (warp == kMmaWarp)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem), "r"(kXCols) : "memory");
+}
+
+// Tiles (halves) a CTA. One CTA fits an SM, and a round of two-tile CTAs takes 1.23 (D = 64),
+// 1.42 (256), 1.64 (512), 1.78 (1,021) or 1.90 (2,500) times a round of one-tile CTAs: two
+// pay where they take nearly half the rounds.  N S = 24,000 (two rounds or one): D = 64
+// 0.129 -> 0.084 ms, 256 0.54 -> 0.39, 512 1.25 -> 1.03, 1,021 3.48 -> 3.13; N S = 65,536
+// (four or two): 2,500 32.4 -> 30.9.
+int x_halves(int64_t N, int S) {
+    constexpr int64_t kSms = 152;
+    const int64_t one = ((N + kXP - 1) / kXP) * S, two = ((N + 2 * kXP - 1) / (2 * kXP)) * S;
+    const int64_t rounds1 = (one + kSms - 1) / kSms, rounds2 = (two + kSms - 1) / kSms;
+    return N > kXP && 10 * rounds1 >= 19 * rounds2 ? 2 : 1;
+}
+// Tiles of 128 points per shift, padded to whole CTAs.
+int64_t x_tiles(int64_t N, int S) {
+    const int64_t w = (int64_t)x_halves(N, S) * kXP;
+    return (N + w - 1) / w * (w / kXP);
+}
+
+template <int H>
+cudaError_t launch_x(const XArgs& a, int ctas, cudaStream_t st) {
+    static std::mutex mu;
+    static std::map<int, bool> attr;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        if (!attr[dev]) {
+            const cudaError_t e = cudaFuncSetAttribute(full_fix_tc_kernel<H>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)sizeof(XSmem<H>));
+            if (e != cudaSuccess) return e;
+            attr[dev] = true;
+        }
+    }
+    full_fix_tc_kernel<H><<<(unsigned)ctas, kXThreads<H>, sizeof(XSmem<H>), st>>>(a);
+    return cudaGetLastError();
 }
 
 size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -456,7 +523,7 @@ size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
 size_t full_fix_tc_scratch_bytes(int64_t D, int64_t N, int S) {
     const int64_t nP = (D + kXB - 1) / kXB, nC = 2 * nP;
     return al((size_t)nP * nC * kXChunkB) + al(sizeof(fix::Digits) * (size_t)nP * kXB * kXB) + al(sizeof(FixVar) * D) +
-           al((size_t)S * ((N + kXP - 1) / kXP) * nC * kXChunkA);
+           al((size_t)S * x_tiles(N, S) * nC * kXChunkA);
 }
 
 cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int64_t N, int S, const uint32_t* g,
@@ -473,25 +540,13 @@ cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int6
     fix_tc_tables_kernel<<<(unsigned)(nP * kXB), 128, 0, st>>>(A, u, (int)D, (int)nC, var, Lb, Lp);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    static std::mutex mu;
-    static std::map<int, bool> attr;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        if (!attr[dev]) {
-            e = cudaFuncSetAttribute(full_fix_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)sizeof(XSmem));
-            if (e != cudaSuccess) return e;
-            attr[dev] = true;
-        }
-    }
     XArgs a;
     a.D = (int)D;
     a.nP = (int)nP;
     a.nC = (int)nC;
     a.N = N;
-    a.tps = (int)((N + kXP - 1) / kXP);
+    const int halves = x_halves(N, S);
+    a.tps = (int)(x_tiles(N, S) / halves);
     a.g = g;
     a.delta = delta;
     a.u = u;
@@ -505,8 +560,7 @@ cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int6
     a.timeout = timeout;
     a.wait_ns = (wait_ns > 0 && wait_ns < kXWaitNs) ? wait_ns : kXWaitNs;
     if (ev_begin && (e = cudaEventRecord(ev_begin, st)) != cudaSuccess) return e;
-    full_fix_tc_kernel<<<(unsigned)(S * a.tps), kXThreads, sizeof(XSmem), st>>>(a);
-    e = cudaGetLastError();
+    e = halves == 2 ? launch_x<2>(a, S * a.tps, st) : launch_x<1>(a, S * a.tps, st);
     if (e == cudaSuccess && ev_end) e = cudaEventRecord(ev_end, st);
     return e;
 }

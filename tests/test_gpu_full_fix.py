@@ -50,6 +50,15 @@ def test_threshold_ranges(ctx, D, deep):
     _check(ctx, s, (1, 1.0, 0.15, 1.5, 0.0), u, 140, 4, 9)
 
 
+@pytest.mark.parametrize("D,N", [(64, 257), (97, 385), (129, 300), (289, 257)])
+def test_two_tiles_a_cta(ctx, D, N):
+    """64 shifts of a few tiles: more tiles than SMs, so a CTA takes two, the second
+    of a shift partly or wholly beyond its points."""
+    s = inputs.uniform_sites(D, 400 + D)
+    u = inputs.rng(D, 1).normal(0.7, 0.4, size=D)
+    _check(ctx, s, (0, 1.1, 0.2, 0.5, 0.0), u, N, 64, D + 1)
+
+
 def test_scratch_limit(ctx):
     """With room for the integer form's history (2.1 GB) but not for the tensor-core
     form's (4.3 GB), the call takes the integer form."""
