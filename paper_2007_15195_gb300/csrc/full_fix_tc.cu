@@ -117,15 +117,6 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* b) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
 }
-__device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(smem_u32(b)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
 __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -491,7 +482,8 @@ int x_halves(int64_t N, int S) {
     const int64_t rounds1 = (one + kSms - 1) / kSms, rounds2 = (two + kSms - 1) / kSms;
     return N > kXP && 10 * rounds1 >= 19 * rounds2 ? 2 : 1;
 }
-// Tiles of 128 points per shift, padded to whole CTAs.
+// Tiles of 128 points per shift, padded to whole CTAs: with N > 128 at most the
+// ceil(N / 64) sums a shift has room for.
 int64_t x_tiles(int64_t N, int S) {
     const int64_t w = (int64_t)x_halves(N, S) * kXP;
     return (N + w - 1) / w * (w / kXP);

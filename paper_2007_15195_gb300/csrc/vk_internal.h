@@ -207,8 +207,8 @@ cudaError_t launch_full_genz_tc(const double* A, const double* u, int64_t D, int
                                 cudaStream_t st);
 
 // The FP64 recursion with its contraction on the tensor cores (full_fix_tc.cu),
-// given the FP64 factor A: part gets part_stride sums per shift, of which it
-// writes the first ceil(N / 128) (the caller zeroes the rest).
+// given the FP64 factor A: part gets part_stride >= ceil(N / 64) sums per shift, of
+// which it writes the first ceil(N / 128), or 2 ceil(N / 256) (the caller zeroes the rest).
 size_t full_fix_tc_scratch_bytes(int64_t D, int64_t N, int S);
 cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int64_t N, int S, const uint32_t* g,
                                const double* delta, int dim, void* scratch, double* part, int part_stride,
