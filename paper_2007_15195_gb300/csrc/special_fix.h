@@ -172,12 +172,14 @@ struct FixFloat {
 
 VK_FIX_FN bool is_tail(const FixProb& p) { return (p.E >> 63) == 0; }
 
-// Phi(z) as mantissa and exponent (within 2^-53 relative from E, else from t).
+// Phi(z) as mantissa and exponent: the tail's own below 1/2, else E.  (E's bits
+// below 1/2 too would leave the mantissa unnormalised, and the product of two such
+// loses the bits that umul_hi drops: 5.6e-13 at z = -3.29 twice.)
 VK_FIX_FN FixFloat prob(const FixProb& p) {
     FixFloat r;
-    const bool tiny = (p.E >> 53) == 0;
-    r.m = tiny ? p.mt : p.E;
-    r.ex = tiny ? p.et : 0;
+    const bool t = is_tail(p);
+    r.m = t ? p.mt : p.E;
+    r.ex = t ? p.et : 0;
     return r;
 }
 
@@ -192,7 +194,7 @@ VK_FIX_FN uint64_t tent(uint64_t X) {
 VK_FIX_FN FixFloat times(FixFloat f, const FixProb& p) {
     FixFloat e = prob(p), r;
     r.m = umul_hi(f.m, e.m);
-    const int k = clz32((uint32_t)(r.m >> 32));  // E >= 2^53, or mt >= 2^62 (or 0: k = 32, the product stays 0)
+    const int k = clz32((uint32_t)(r.m >> 32));  // f.m and e.m >= 2^62 (or 0: k = 32, the product stays 0)
     r.m <<= k;
     r.ex = f.ex + e.ex + k;
     return r;
