@@ -109,16 +109,7 @@ __device__ __forceinline__ fix::Digits fix_quantile(const fix::FixTables& tb, ui
 // Phi of the conditional mean whose product with rdiag is hi.
 __device__ __forceinline__ void fix_phi(const fix::FixTables& tb, int64_t hi, int64_t lim, int shift, fix::FixProb& e,
                                         uint64_t K) {
-    const int64_t neg = hi >> 63;
-    const int64_t a = (hi ^ neg) - neg;
-    const uint64_t A = (uint64_t)a << (shift & 63);  // |z| 2^58
-    const bool big = a >= lim;
-    uint64_t T;
-    fix::tail_poly(tb.tail, tb.meta, A, e.mt, e.et, K);
-    T = e.mt >> e.et;
-    if (big) e.mt = T = 0;  // z >= 9.25: Phi = 1 to 2^-66
-    e.E = T ^ (uint64_t)~neg;
-    if (hi < 0 && (big || A >= (7ull << 58))) deep_prob(hi, shift, e);
+    if (fix::phi_of(tb.tail, tb.meta, hi, lim, shift, e, K)) deep_prob(hi, shift, e);
 }
 
 }  // namespace vk

@@ -156,6 +156,17 @@ VK_FIX_FN int64_t poly(const FixRow& r, Digits X, int shift3, uint64_t K) {
     return mul_add(digits(P), X, r.c0, K);
 }
 
+// v >> n for n >= 0, 0 from n = 64 on (PTX's shift clamps its amount; C++'s is undefined there).
+VK_FIX_FN uint64_t shr64(uint64_t v, int n) {
+#ifdef __CUDA_ARCH__
+    uint64_t r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
+#else
+    return n < 64 ? v >> n : 0;
+#endif
+}
+
 // Phi(z): E its Q0.64 value (below 2^63 exactly where it is taken as the
 // tail t = Phi(-|z|), above as 1 - t), and t = mt 2^-64 2^-et (mt = 0: none)
 // for the places where E's last bit is not relative accuracy enough.
@@ -200,7 +211,6 @@ VK_FIX_FN FixFloat times(FixFloat f, const FixProb& p) {
     return r;
 }
 
-VK_FIX_FN uint64_t shr64(uint64_t v, int n) { return n < 64 ? v >> n : 0; }
 
 // s = min(w e, 1 - w e) where it is below 2^-11, from the operands' mantissas
 // and exponents: s = m 2^-64 2^-lz, m >= 2^63 (0 when s is 0).
@@ -247,6 +257,22 @@ VK_FIX_FN void tail_poly(const FixRow* rows, const uint16_t* meta, uint64_t A, u
     const int w = meta[i];
     mt = (uint64_t)poly(rows[i], X, w & 255, K) << 2;
     et = w >> 8;
+}
+
+// Phi of z = hi 2^(shift - 58), lim the value of |hi| at |z| = 9.25, for z > -7; true
+// where z is below that and the FP64 tail takes over.
+VK_FIX_FN bool phi_of(const FixRow* rows, const uint16_t* meta, int64_t hi, int64_t lim, int shift, FixProb& e,
+                      uint64_t K) {
+    const int64_t neg = hi >> 63;
+    const int64_t a = (hi ^ neg) - neg;
+    const uint64_t A = (uint64_t)a << (shift & 63);  // |z| 2^58
+    const bool big = a >= lim;
+    uint64_t T;
+    tail_poly(rows, meta, A, e.mt, e.et, K);
+    T = shr64(e.mt, e.et);
+    if (big) e.mt = T = 0;  // z >= 9.25: Phi = 1 to 2^-66
+    e.E = T ^ (uint64_t)~neg;
+    return hi < 0 && (big || A >= (7ull << 58));
 }
 
 // A non-negative finite double below 1 as mantissa and exponent (0: m = 0).
