@@ -779,6 +779,20 @@ void mixture_nodes(int n, double beta, double gamma, std::vector<double>& r, std
 
 // ------------------------------ host ordering ------------------------------
 
+// floor(t) kept in [0, 2^30], NaN as 0 (the device's rule: knn.cu, quantise).
+int64_t quantised(double t) {
+    return t >= 1073741824.0 ? (int64_t)1 << 30 : t > 0.0 ? (int64_t)std::floor(t) : 0;
+}
+
+// Order-preserving integer image of a double (-0 as +0; NaN beyond the infinities), so
+// that a sort has a total order whatever the values.
+uint64_t ord_key(double x) {
+    uint64_t b;
+    if (x == 0.0) x = 0.0;
+    std::memcpy(&b, &x, sizeof b);
+    return (b >> 63) ? ~b : (b | 0x8000000000000000ULL);
+}
+
 void quantize_host(const double* s, int64_t D, std::vector<int64_t>& q) {
     q.assign(2 * (size_t)D, 0);
     double x0 = s[0], x1 = s[0], y0 = s[1], y1 = s[1];
@@ -795,8 +809,8 @@ void quantize_host(const double* s, int64_t D, std::vector<int64_t>& q) {
     for (int64_t i = 0; i < D; ++i) {
         const double tx = s[2 * i] - x0;
         const double ty = s[2 * i + 1] - y0;
-        q[2 * (size_t)i] = (int64_t)std::floor(tx * c);
-        q[2 * (size_t)i + 1] = (int64_t)std::floor(ty * c);
+        q[2 * (size_t)i] = quantised(tx * c);
+        q[2 * (size_t)i + 1] = quantised(ty * c);
     }
 }
 
@@ -1007,9 +1021,10 @@ int vecchia_order(vecchia_ctx* c, const double* sites, int64_t D, int kind, int3
     for (int64_t i = 0; i < D; ++i) p[(size_t)i] = (int32_t)i;
     if (kind == VECCHIA_ORDER_XY) {
         std::sort(p.begin(), p.end(), [s](int32_t a, int32_t b) {
-            if (s[2 * a] != s[2 * b]) return s[2 * a] < s[2 * b];
-            if (s[2 * a + 1] != s[2 * b + 1]) return s[2 * a + 1] < s[2 * b + 1];
-            return a < b;
+            const uint64_t xa = ord_key(s[2 * (int64_t)a]), xb = ord_key(s[2 * (int64_t)b]);
+            if (xa != xb) return xa < xb;
+            const uint64_t ya = ord_key(s[2 * (int64_t)a + 1]), yb = ord_key(s[2 * (int64_t)b + 1]);
+            return ya != yb ? ya < yb : a < b;
         });
     } else if (kind == VECCHIA_ORDER_MAXMIN) {
         order_maxmin(s, D, p.data());

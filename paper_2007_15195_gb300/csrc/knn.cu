@@ -74,9 +74,14 @@ __device__ __forceinline__ Grid box_grid(const unsigned long long (&k)[4], int g
     return g;
 }
 
+// Coordinates index cells, so they are kept in [0, 2^30] where the box does not
+// bound them: a NaN leaves its axis out of the extent, and an extent below 2^-994
+// makes c infinite.  (The host ordering's rule, too.)
 __device__ __forceinline__ int2 quantise(const Grid& g, double x, double y) {
     if (g.zero) return make_int2(0, 0);
-    return make_int2((int)floor(__dmul_rn(__dsub_rn(x, g.xmin), g.c)), (int)floor(__dmul_rn(__dsub_rn(y, g.ymin), g.c)));
+    const int qx = __double2int_rd(__dmul_rn(__dsub_rn(x, g.xmin), g.c));
+    const int qy = __double2int_rd(__dmul_rn(__dsub_rn(y, g.ymin), g.c));
+    return make_int2(min(max(qx, 0), 1 << 30), min(max(qy, 0), 1 << 30));
 }
 
 // Bounding box of the sites: maxima of the keys of x, y and of their
