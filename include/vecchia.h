@@ -395,17 +395,20 @@ int vecchia_set_timing(vecchia_ctx* ctx, int enable);
 /* Milliseconds between those events in the last call with timing on. */
 int vecchia_genz_time_ms(const vecchia_ctx* ctx, double* ms);
 
-/* Bounded device waits of vecchia_full_genz's tensor-core recursion (mixed
- * precision; the paper has no counterpart: this is how the library reports a
- * stalled kernel instead of hanging).  Its point warps wait on mbarriers for
- * the accumulators and its copy lane for their progress; a wait with no
- * progress for limit_ns (0 = the built-in 2 s; values above it are clamped
- * to it) makes the kernel record a timeout, wait (with the full 2 s limit)
- * for every copy and MMA it has issued, free its tensor memory and return,
- * and the call then returns VECCHIA_ERR_TIMEOUT.  withhold != 0 is for tests
- * of that path only: the copy lane issues no copy and no MMA, so the first
- * accumulator wait runs out with nothing in flight.  The setting stays on the
- * context until changed; (0, 0) restores the default. */
+/* Bounded device waits of vecchia_full_genz's tensor-core recursions (the
+ * paper has no counterpart: this is how the library reports a stalled kernel
+ * instead of hanging).  Their point warps wait on mbarriers for the
+ * accumulators, their copy (and, FP64 from 64 variables on, MMA) lanes for
+ * progress; a wait with no progress for the limit makes the kernel record a
+ * timeout, wait (with the full 2 s limit) for every copy and MMA it has
+ * issued, free its tensor memory and return, and the call then returns
+ * VECCHIA_ERR_TIMEOUT.  limit_ns is the limit of the mixed precision's
+ * recursion (0 = the built-in 2 s; values above it are clamped to it); the
+ * FP64 recursion keeps 2 s.  withhold != 0 is for tests of that path only: the
+ * mixed recursion's copy lane issues no copy and no MMA, so the first
+ * accumulator wait runs out with nothing in flight; with bit 1 set (2), limit_ns
+ * and the withholding hold for the FP64 recursion as well.  The setting stays
+ * on the context until changed; (0, 0) restores the default. */
 int vecchia_set_full_genz_wait(vecchia_ctx* ctx, uint64_t limit_ns, int withhold);
 
 /* Diagnostic: the FP32 special functions of the mixed path on n values (x and

@@ -566,9 +566,10 @@ def vecchia_set_timing(ctx, enable=True):
 
 
 def vecchia_set_full_genz_wait(ctx, limit_ns=0, withhold=False):
-    """Wait limit of the tensor-core full-Genz kernel (0 = built-in 2 s) and
-    the test switch that makes its copy lane issue nothing."""
-    _check(lib().vecchia_set_full_genz_wait(ctx.handle, C.c_uint64(int(limit_ns)), 1 if withhold else 0),
+    """Wait limit of the mixed full-Genz kernel (0 = built-in 2 s) and the test
+    switch that makes its copy lane issue nothing (2: limit and switch for the
+    FP64 kernel, too)."""
+    _check(lib().vecchia_set_full_genz_wait(ctx.handle, C.c_uint64(int(limit_ns)), int(withhold or 0)),
            "vecchia_set_full_genz_wait", ctx)
 
 

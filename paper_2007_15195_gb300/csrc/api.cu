@@ -2020,7 +2020,7 @@ int vecchia_genz_time_ms(const vecchia_ctx* c, double* ms) {
 int vecchia_set_full_genz_wait(vecchia_ctx* c, uint64_t limit_ns, int withhold) {
     if (!c) return VECCHIA_ERR_ARG;
     c->full_wait_ns = limit_ns;
-    c->full_withhold = withhold ? 1 : 0;
+    c->full_withhold = withhold;
     return VECCHIA_OK;
 }
 

@@ -852,8 +852,8 @@ cudaError_t launch_full_genz(const double* sites, const double* u, int64_t D, co
     } else if (tc64) {
         e = cudaMemsetAsync(part, 0, sizeof(double) * S * nblk, st);
         if (e == cudaSuccess)
-            e = launch_full_fix_tc(A, u, D, N, S, gdev, delta, (int)dim, p, part, (int)nblk, bad + 1, wait_ns, ev_begin,
-                                   ev_end, st);
+            e = launch_full_fix_tc(A, u, D, N, S, gdev, delta, (int)dim, p, part, (int)nblk, bad + 1,
+                                   (withhold & 2) ? wait_ns : 0, (withhold & 2) != 0, ev_begin, ev_end, st);
     } else {
         void* Ld = p;
         p += al(sizeof(fix::Digits) * D * D);

@@ -100,6 +100,7 @@ struct XArgs {
     int part_stride;
     int* timeout;
     uint64_t wait_ns;
+    int withhold;               // tests: the copy lane issues nothing
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -255,6 +256,7 @@ __device__ void copy_all(const XArgs& a, XSmem<H>& sm, const unsigned char* Yt) 
     constexpr int ST = kXStages<H>;
     int il = 0, seen[H] = {};  // copies issued; panels whose y a half's points have written
     bool ok = true;
+    if (a.withhold) return;
     for (int p = 1; p < a.nP && ok; ++p)
         for (int c0 = 0; c0 < 2 * p && ok; c0 += kXGroup)
 #pragma unroll
@@ -520,7 +522,8 @@ size_t full_fix_tc_scratch_bytes(int64_t D, int64_t N, int S) {
 
 cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int64_t N, int S, const uint32_t* g,
                                const double* delta, int dim, void* scratch, double* part, int part_stride,
-                               int* timeout, uint64_t wait_ns, cudaEvent_t ev_begin, cudaEvent_t ev_end, cudaStream_t st) {
+                               int* timeout, uint64_t wait_ns, bool withhold, cudaEvent_t ev_begin, cudaEvent_t ev_end,
+                               cudaStream_t st) {
     const int64_t nP = (D + kXB - 1) / kXB, nC = 2 * nP;
     char* p = (char*)scratch;
     unsigned char* Lb = (unsigned char*)p;
@@ -551,6 +554,7 @@ cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int6
     a.part_stride = part_stride;
     a.timeout = timeout;
     a.wait_ns = (wait_ns > 0 && wait_ns < kXWaitNs) ? wait_ns : kXWaitNs;
+    a.withhold = withhold;
     if (ev_begin && (e = cudaEventRecord(ev_begin, st)) != cudaSuccess) return e;
     e = halves == 2 ? launch_x<2>(a, S * a.tps, st) : launch_x<1>(a, S * a.tps, st);
     if (e == cudaSuccess && ev_end) e = cudaEventRecord(ev_end, st);

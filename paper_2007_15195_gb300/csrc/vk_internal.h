@@ -189,8 +189,8 @@ size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed, bool tc6
 int64_t full_genz_blocks_per_shift(int64_t N, bool mixed);
 // part_host: per-shift point-block sums (S x full_genz_blocks_per_shift); bad_host:
 // the first failing pivot (INT_MAX if none); timeout_host: nonzero if a device
-// wait of the tensor-core kernel ran out; ev_begin / ev_end (may be null) are
-// recorded around the recursion kernel alone.
+// wait of a tensor-core kernel ran out; wait_ns, withhold: vecchia_set_full_genz_wait's;
+// ev_begin / ev_end (may be null) are recorded around the recursion kernel alone.
 cudaError_t launch_full_genz(const double* sites, const double* u, int64_t D, const vecchia_cov& cov, int64_t N,
                              int S, bool mixed, bool tc64, const uint32_t* g_host, const uint32_t* gfix_host,
                              uint64_t seed, void* scratch, double* part_host, int* bad_host, int* timeout_host,
@@ -208,11 +208,12 @@ cudaError_t launch_full_genz_tc(const double* A, const double* u, int64_t D, int
 
 // The FP64 recursion with its contraction on the tensor cores (full_fix_tc.cu),
 // given the FP64 factor A: part gets part_stride >= ceil(N / 64) sums per shift, of
-// which it writes the first ceil(N / 128), or 2 ceil(N / 256) (the caller zeroes the rest).
+// which it writes the first ceil(N / 128), or 2 ceil(N / 256) (the caller zeroes the rest);
+// wait_ns and withhold as for the mixed form.
 size_t full_fix_tc_scratch_bytes(int64_t D, int64_t N, int S);
 cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int64_t N, int S, const uint32_t* g,
                                const double* delta, int dim, void* scratch, double* part, int part_stride,
-                               int* timeout, uint64_t wait_ns, cudaEvent_t ev_begin, cudaEvent_t ev_end,
+                               int* timeout, uint64_t wait_ns, bool withhold, cudaEvent_t ev_begin, cudaEvent_t ev_end,
                                cudaStream_t st);
 
 // sites_out[k] = sites[perm[k]], u_out[k] = u[perm[k]]; *bad = 1 on an index out of range.
