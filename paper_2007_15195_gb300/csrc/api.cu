@@ -1099,9 +1099,10 @@ int vecchia_log_cdf_unordered(vecchia_ctx* c, const double* sites, const double*
     const size_t o_bad = dv.off;
     dv.take<int>(1);
     const size_t o_scr = dv.off;
-    dv.take<char>(std::max(std::max(vk::knn_scratch_bytes(D), vk::order_xy_scratch_bytes(D)),
-                           order_kind == VECCHIA_ORDER_MAXMIN ? vk::maxmin_scratch_bytes(D) : (size_t)0));
-    int st = ensure_aux(c, dv.off);
+    dv.take<char>(std::max(vk::knn_scratch_bytes(D), order_kind == VECCHIA_ORDER_MAXMIN ? vk::maxmin_scratch_bytes(D) : 0));
+    // the XY order's scratch is over before the ordered copies and the rows are written: it takes their place
+    const size_t xy = order_kind == VECCHIA_ORDER_XY ? vk::order_xy_scratch_bytes(D) : 0;
+    int st = ensure_aux(c, std::max(dv.off, o_so + xy));
     if (st != VECCHIA_OK) return st;
     char* X = (char*)c->aux;
     const cudaStream_t s = c->stream;
@@ -1126,7 +1127,7 @@ int vecchia_log_cdf_unordered(vecchia_ctx* c, const double* sites, const double*
         if (order_kind == VECCHIA_ORDER_MAXMIN) {
             e = vk::launch_maxmin(sd, D, perm, X + o_scr, s);
         } else if (order_kind == VECCHIA_ORDER_XY) {
-            e = vk::launch_order_xy(sd, D, perm, X + o_scr, s);
+            e = vk::launch_order_xy(sd, D, perm, X + o_so, s);
         } else {
             hp.resize((size_t)D);
             for (int64_t k = 0; k < D; ++k) hp[(size_t)k] = (int32_t)k;

@@ -736,25 +736,10 @@ __global__ void sort_merge_kernel(SortRun in, SortRun out, int D, int64_t w, int
     }
 }
 
-size_t sort_scratch_bytes(int64_t D, bool two) {
-    return 2 * (align256(8 * (size_t)D) * (two ? 2 : 1) + align256(4 * (size_t)D));
-}
-
+// r: two sets of D entries, the first of which may lie where KEYS reads its own
+// (a tile is read whole before it is written).
 template <bool TWO, class KEYS>
-cudaError_t launch_sort(KEYS keys, int64_t D, int32_t* perm, void* scratch, cudaStream_t st) {
-    SortRun r[2];
-    char* p = (char*)scratch;
-    for (int k = 0; k < 2; ++k) {
-        r[k].a = (unsigned long long*)p;
-        p += align256(8 * (size_t)D);
-        r[k].b = nullptr;
-        if (TWO) {
-            r[k].b = (unsigned long long*)p;
-            p += align256(8 * (size_t)D);
-        }
-        r[k].idx = (int*)p;
-        p += align256(4 * (size_t)D);
-    }
+cudaError_t launch_sort(KEYS keys, int64_t D, int32_t* perm, const SortRun (&r)[2], cudaStream_t st) {
     const int tiles = (int)((D + kSortTile - 1) / kSortTile);
     sort_tile_kernel<TWO><<<tiles, kSortTile / 2, 0, st>>>(keys, (int)D, r[0], tiles == 1 ? perm : nullptr);
     int cur = 0;
@@ -1160,7 +1145,7 @@ struct MmKeys {  // descending key, then ascending index
 
 size_t maxmin_scratch_bytes(int64_t D) {
     return knn_scratch_bytes(D) + 2 * align256(sizeof(long long) * (size_t)D) + 2 * align256(sizeof(int) * (size_t)D) +
-           align256(sizeof(MmSlot) * 3 * kMmMaxCluster + (3 + kMmRounds) * sizeof(int)) + sort_scratch_bytes(D, false);
+           align256(sizeof(MmSlot) * 3 * kMmMaxCluster + (3 + kMmRounds) * sizeof(int));
 }
 
 // The largest cluster that the device schedules (16 is beyond the portable 8).
@@ -1208,7 +1193,6 @@ cudaError_t launch_maxmin(const double* sites, int64_t D, int32_t* perm, void* s
     p += align256(sizeof(int) * (size_t)D);
     S.slot = (MmSlot*)p;
     S.count = (int*)(p + sizeof(MmSlot) * 3 * kMmMaxCluster);
-    p += align256(sizeof(MmSlot) * 3 * kMmMaxCluster + (3 + kMmRounds) * sizeof(int));
     e = cudaMemsetAsync(S.count, 0, (3 + kMmRounds) * sizeof(int), st);
     if (e != cudaSuccess) return e;
     int dev = 0;
@@ -1237,7 +1221,9 @@ cudaError_t launch_maxmin(const double* sites, int64_t D, int32_t* perm, void* s
     }
     e = cudaLaunchKernelEx(&cfg, maxmin_kernel, (const Grid*)c.grid, S, (int)D, rounds == 0, true, rounds);
     if (e != cudaSuccess) return e;
-    return launch_sort<false>(MmKeys{S.key, S.pts}, D, perm, p, st);
+    // the sort's runs take the place of what the rounds leave behind (keys in place)
+    const SortRun runs[2] = {{(unsigned long long*)S.key, nullptr, S.list}, {(unsigned long long*)S.mind, nullptr, S.wit}};
+    return launch_sort<false>(MmKeys{S.key, S.pts}, D, perm, runs, st);
 }
 
 // ---- XY ordering on the device ------------------------------------------------
@@ -1290,12 +1276,22 @@ struct XyKeys {
 };
 
 size_t order_xy_scratch_bytes(int64_t D) {
-    return D > kXyMax ? sort_scratch_bytes(D, true) : sizeof(int) * (size_t)(D > 0 ? D : 1);
+    return D > kXyMax ? 2 * (2 * align256(8 * (size_t)D) + align256(4 * (size_t)D)) : sizeof(int) * (size_t)(D > 0 ? D : 1);
 }
 
 cudaError_t launch_order_xy(const double* sites, int64_t D, int32_t* perm, void* scratch, cudaStream_t st) {
     if (D <= 0 || D > INT_MAX / 2) return cudaErrorInvalidValue;
-    if (D > kXyMax) return launch_sort<true>(XyKeys{sites}, D, perm, scratch, st);
+    if (D > kXyMax) {
+        SortRun r[2];
+        char* p = (char*)scratch;
+        for (SortRun& k : r) {
+            k.a = (unsigned long long*)p;
+            k.b = (unsigned long long*)(p + align256(8 * (size_t)D));
+            k.idx = (int*)(p + 2 * align256(8 * (size_t)D));
+            p += 2 * align256(8 * (size_t)D) + align256(4 * (size_t)D);
+        }
+        return launch_sort<true>(XyKeys{sites}, D, perm, r, st);
+    }
     int* rank = (int*)scratch;
     cudaError_t e = cudaMemsetAsync(rank, 0, sizeof(int) * (size_t)D, st);
     if (e != cudaSuccess) return e;
