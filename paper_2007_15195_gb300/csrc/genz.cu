@@ -521,9 +521,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 // Work items: (problem, site, shift group).  A list of segments maps a flat
 // item index to them: segment k covers items [seg_prefix[k], seg_prefix[k+1])
 // = sites seg_base[k].y, ... of problem seg_base[k].x, each split into
-// `groups` shift groups (the group index varies fastest).  With an explicit
-// `items` list (the FP64 re-evaluation of flagged sites) an item is
-// (problem, site) with all shifts, and its count may live on the device.
+// `groups` shift groups (the group index varies fastest).  The log-space form
+// takes an explicit list of (problem, site) instead, its count on the device.
 //
 // The last round of a launch: with items of equal size, a launch of n items
 // on a grid of G CTAs leaves n mod G CTAs with one item more than the rest,
@@ -533,8 +532,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 // that spread over the whole grid.  A shift's partial means are computed by
 // one warp whatever the grouping, so the results do not change.
 struct ItemSrc {
-    const int2* items;       // explicit (problem, site) items, or nullptr
-    const int* dev_count;    // device-side count for `items`, or nullptr
+    const int2* items;       // the log-space form's (problem, site) list, or nullptr
+    const int* dev_count;    // its device-side count
     const int* seg_prefix;   // n_segs + 1 prefix sums of items
     const int2* seg_base;    // (problem, first site) per segment
     int n_segs;
@@ -546,12 +545,6 @@ struct ItemSrc {
 };
 
 __device__ __forceinline__ void item_of(const ItemSrc& src, int it, int2& ps, int& grp, int& ngroups) {
-    if (src.items) {
-        ps = src.items[it];
-        grp = 0;
-        ngroups = 1;
-        return;
-    }
     int site_item;
     const int whole = src.whole_sites * src.groups;
     if (it < whole) {
@@ -573,6 +566,16 @@ __device__ __forceinline__ void item_of(const ItemSrc& src, int it, int2& ps, in
             hi = mid - 1;
     }
     ps = make_int2(src.seg_base[lo].x, src.seg_base[lo].y + (site_item - src.seg_prefix[lo]));
+}
+
+// Entry and shift group of item `it` of the explicit list: the entries before `whole`
+// with all shifts, the others in tail_groups.
+__device__ __forceinline__ void listed_item_of(const ItemSrc& src, int whole, int tail_groups, int it, int2& ps,
+                                               int& grp, int& ngroups) {
+    const int j = it - whole, k = j < 0 ? 0 : j / tail_groups;
+    ngroups = j < 0 ? 1 : tail_groups;
+    grp = j < 0 ? 0 : j - k * tail_groups;
+    ps = src.items[j < 0 ? it : whole + k];
 }
 
 // MODE: 0 = FP64, 1 = mixed fast form, 2 = mixed log-space form.
@@ -655,11 +658,31 @@ __device__ __forceinline__ bool term_block(GenzSmem<DMAX, MIXED>& sm, const Prob
 // N alone (so a problem's sums do not depend on the batch it runs in): one in the
 // mixed fast form, whose FP32 lane sums another split would round anew; FP64 as
 // many as make the units (shifts x slices) a multiple of four warps; four in the
-// log-space form, whose few flagged terms run one to a CTA.
+// log-space form, a unit for each of its four warps.
 __host__ __device__ constexpr int auto_slices(int S, int64_t N, int mode) {
     int g = mode == kModeFast ? 1 : (mode == kModeSafe || (S & 1)) ? 4 : (S & 2) ? 2 : 1;
     while (g > 1 && (S * g > kMaxUnits || N < 256 * g)) g >>= 1;
     return g;
+}
+
+// Shift groups for the `rest` entries of the list's last round on a grid of G CTAs (all
+// entries, where there are fewer than CTAs): of 1, 2, 4, ... the number whose rounds
+// take the fewest steps, an item's being its factor (about 3 a variable and 20) and its
+// warps' rounds of units.  Any listed problem may stand for the rest: the groups do not
+// change a shift's sums.
+__device__ __forceinline__ int listed_groups(const ProbDev& P, int rest, int G, int max_S, int slices, int n_warps) {
+    const int64_t unit = (P.N + 32 * slices - 1) / (32 * slices) * (P.m + 1);
+    int64_t best = LLONG_MAX;
+    int groups = 1;
+    for (int g = 1; g <= max_S; g *= 2) {
+        const int units = (max_S + g - 1) / g * slices;
+        const int64_t t = ((int64_t)rest * g + G - 1) / G * (3 * P.m + 20 + (units + n_warps - 1) / n_warps * unit);
+        if (t < best) {
+            best = t;
+            groups = g;
+        }
+    }
+    return groups;
 }
 
 template <int DMAX, int P, int MODE>
@@ -678,11 +701,23 @@ __global__ void __launch_bounds__(max_threads(DMAX, P, MODE)) __maxnreg__(reg_ca
         load_fix_tables(fix_tables<DMAX>());
         __syncthreads();
     }
-    const int n_run = src.dev_count ? min(*src.dev_count, src.n_items) : src.n_items;
+    int n_run = src.n_items, whole = 0, tail_groups = 1;
+    if constexpr (MODE == kModeSafe) {
+        const int n = min(*src.dev_count, src.n_items), G = (int)gridDim.x;
+        whole = n / G * G;
+        if (n > whole) {
+            const ProbDev& P0 = probs[src.items[whole].x];
+            tail_groups = listed_groups(P0, n - whole, G, max_S, auto_slices(P0.S, P0.N, MODE), n_warps);
+        }
+        n_run = whole + (n - whole) * tail_groups;
+    }
     for (int it = blockIdx.x; it < n_run; it += gridDim.x) {
         int2 item;
         int grp, groups;
-        item_of(src, it, item, grp, groups);
+        if constexpr (MODE == kModeSafe)
+            listed_item_of(src, whole, tail_groups, it, item, grp, groups);
+        else
+            item_of(src, it, item, grp, groups);
         const ProbDev& Pd = probs[item.x];
         const int64_t term = item.y;
         const int S = Pd.S;
@@ -1266,16 +1301,20 @@ cudaError_t launch_genz(int bucket, bool mixed, const GenzTile& tile, const Prob
 #undef VK_ARGS
 }
 
+// The flagged terms: four warps a CTA (eight above 32 variables), each shift in four
+// slices, several CTAs an SM, so that one term's factor runs beside the others' points;
+// the last round's terms (all, where few are flagged) in shift groups over the whole
+// grid.  2,500 terms, all flagged, whole call in ms, against 16 warps a term, one CTA an
+// SM: m = 20, N S = 256 x 8 1.04 against 1.54, 2,048 x 8 5.46 against 5.59, 4,096 x 16 21.5
+// against 21.3; about 100 flagged: 0.50 both, 2.09 against 2.08, 7.70 against 7.68.
 cudaError_t launch_genz_fallback(int max_bucket, const ProbDev* probs, const int* fallback_count,
                                  const int2* fallback_items, int capacity, ProbResult* results,
                                  int max_S, cudaStream_t st) {
     if (capacity <= 0) return cudaSuccess;
-    // 16 warps a term (8 above 32 variables): its shifts in four slices each
-    GenzTile t{16, 1, 0, 1};
     ItemSrc src{fallback_items, fallback_count, nullptr, nullptr, 0, capacity, 1, 0, 1, 0};
     if (max_bucket >= 7)  // blocks of more than 32 variables in the batch
-        return launch_one<64, 1, kModeSafe>(t, probs, src, max_S, results, nullptr, nullptr, st);
-    return launch_one<32, 1, kModeSafe>(t, probs, src, max_S, results, nullptr, nullptr, st);
+        return launch_one<64, 1, kModeSafe>(GenzTile{8, 1, 0, 1}, probs, src, max_S, results, nullptr, nullptr, st);
+    return launch_one<32, 1, kModeSafe>(GenzTile{4, 1, 0, 1}, probs, src, max_S, results, nullptr, nullptr, st);
 }
 
 cudaError_t launch_logsum(const ProbDev* probs, int n_probs, int max_slices, ProbResult* results,
