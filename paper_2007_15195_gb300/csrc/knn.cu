@@ -275,6 +275,10 @@ __device__ __forceinline__ unsigned long long qdist2(int ax, int ay, int bx, int
 }
 
 constexpr int kSearchWarps = 4;
+// An own cell of more sites is searched by itself: 100,000 sites on a line, m = 30, 0.92 ->
+// 0.71 ms; without the rule for m > 32 1.24 -> 1.31, with it 0.91.  (24 to 256 alike;
+// cells of an even spread hold 2 to 8.)
+constexpr int kCrowdedCell = 64;
 
 // One warp per site i: the min(m, lim) nearest sites j < lim, lim = i
 // (group 0) or the first site of i's group of `group` sites.
@@ -305,9 +309,9 @@ __global__ void __launch_bounds__(32 * kSearchWarps) search_kernel(
         if (K == 2 && q > 32) src = L[K - 1];
         return shfl_key(src, (q - 1) & 31);
     };
-    // stage the lanes' candidates that beat the current q-th best; merge full chunks
+    Key w = inf_key();  // the current q-th best (it changes with a merge only)
+    // stage the lanes' candidates that beat it; merge full chunks
     auto offer = [&](bool valid, Key k) {
-        const Key w = worst();
         valid = valid && key_less(k, w);
         const unsigned mask = __ballot_sync(0xffffffffu, valid);
         if (valid) st[n + __popc(mask & ((1u << lane) - 1u))] = k;
@@ -318,6 +322,7 @@ __global__ void __launch_bounds__(32 * kSearchWarps) search_kernel(
             __syncwarp();
             if (lane < n - 32) st[lane] = st[32 + lane];
             n -= 32;
+            w = worst();
             __syncwarp();
         }
     };
@@ -326,6 +331,7 @@ __global__ void __launch_bounds__(32 * kSearchWarps) search_kernel(
             const Key c = (lane < n) ? st[lane] : inf_key();
             merge_chunk<K>(L, c, lane);
             n = 0;
+            w = worst();
             __syncwarp();
         }
     };
@@ -365,22 +371,39 @@ __global__ void __launch_bounds__(32 * kSearchWarps) search_kernel(
                 offer(valid, k);
             }
         };
-        // rings 0 and 1 together (few cells hold q sites, and a merge of a part
-        // chunk costs as much as a full one), then ring by ring, each row of cells as
-        // one run of candidates (100,000 sites in maxmin order, m = 30: 657 -> 400 us)
-        for (int r = 1;; ++r) {
-            if (r == 1) {
-                for (int cy = cy0 - 1; cy <= cy0 + 1; ++cy) cells(cy, cx0 - 1, cx0 + 1);
-            } else {
-                cells(cy0 - r, cx0 - r, cx0 + r);
-                for (int cy = cy0 - r + 1; cy < cy0 + r; ++cy) {
-                    cells(cy, cx0 - r, cx0 - r);
-                    cells(cy, cx0 + r, cx0 + r);
+        // Rings 0 and 1 together (few cells hold q sites, and a merge of a part
+        // chunk costs as much as a full one), a crowded own cell by itself, whose sites
+        // bound the list before the others are offered; then ring by ring, each row of
+        // cells as one run of candidates (100,000 sites in maxmin order, m = 30: 657 -> 400 us).
+        const int own = cy0 * W + cx0;
+        const bool crowded = offsets[own + 1] - offsets[own] > kCrowdedCell;
+        for (int r = crowded ? 0 : 1;; ++r) {
+            const bool rows = r == 0 || (r == 1 && !crowded);  // whole rows, or the ring alone
+            if constexpr (K == 1) {
+                if (rows) {
+                    for (int cy = cy0 - r; cy <= cy0 + r; ++cy) cells(cy, cx0 - r, cx0 + r);
+                } else {
+                    cells(cy0 - r, cx0 - r, cx0 + r);
+                    for (int cy = cy0 - r + 1; cy < cy0 + r; ++cy) {
+                        cells(cy, cx0 - r, cx0 - r);
+                        cells(cy, cx0 + r, cx0 + r);
+                    }
+                    cells(cy0 + r, cx0 - r, cx0 + r);
                 }
-                cells(cy0 + r, cx0 - r, cx0 + r);
+            } else {
+                // one call site, whose body is inlined once, for every run (100,000 normal sites,
+                // m = 50: 0.88 ms, 1.29 with the five above; m = 30 0.70 against 0.55)
+                const int runs = rows ? 2 * r + 1 : 4 * r;
+                for (int t = 0; t < runs; ++t) {
+                    int cy = cy0 - r + t, xa = cx0 - r, xb = cx0 + r;
+                    if (!rows) {  // top and bottom, then the two ends of each row between
+                        cy = t == 0 ? cy0 - r : t == 1 ? cy0 + r : cy0 - r + (t >> 1);
+                        if (t > 1) xa = xb = (t & 1) ? xb : xa;
+                    }
+                    cells(cy, xa, xb);
+                }
             }
             flush();
-            const Key w = worst();
             if (w.d2 != kInfD2) {
                 const long long bound = (long long)r * cs + 1;
                 if (w.d2 < (unsigned long long)(bound * bound)) break;
