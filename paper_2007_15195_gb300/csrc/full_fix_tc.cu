@@ -42,15 +42,12 @@
 #include <mutex>
 
 #include "fix_step.cuh"
+#include "full_fix_plan.h"
 #include "vk_internal.h"
 
 namespace vk {
 namespace {
 
-constexpr int kXP = 128;       // lattice points per tile = MMA M
-constexpr int kXB = 32;        // panel width = MMA N
-constexpr int kXK = 16;        // history chunk (variables) = MMA K
-constexpr int kXDig = 8;       // digits
 constexpr int kXGroup = 8;     // chunks per accumulation
 // H halves of 128 points a CTA (1 or 2): stages of the ring, threads (point warps, the MMA
 // warp, the copy warp)
@@ -58,9 +55,6 @@ template <int H>
 constexpr int kXStages = H == 1 ? 3 : 2;
 template <int H>
 constexpr int kXThreads = H * kXP + 64;
-constexpr uint32_t kRowGroup = kXDig * 256;               // 8 rows: eight 256-byte digit matrices
-constexpr uint32_t kXChunkA = (kXP / 8) * kRowGroup;      // 32,768
-constexpr uint32_t kXChunkB = (kXB / 8) * kRowGroup;      // 8,192
 constexpr uint32_t kXStage = kXChunkA + kXChunkB;
 constexpr uint32_t kXCols = 512;                          // 2 sets x 8 significances x 32
 constexpr uint64_t kXWaitNs = 2000000000ull;
@@ -473,24 +467,6 @@ __global__ void __launch_bounds__(kXThreads<H>, 1) full_fix_tc_kernel(XArgs a) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem), "r"(kXCols) : "memory");
 }
 
-// Tiles (halves) a CTA. One CTA fits an SM, and a round of two-tile CTAs takes 1.23 (D = 64),
-// 1.42 (256), 1.64 (512), 1.78 (1,021) or 1.90 (2,500) times a round of one-tile CTAs: two
-// pay where they take nearly half the rounds.  N S = 24,000 (two rounds or one): D = 64
-// 0.129 -> 0.084 ms, 256 0.54 -> 0.39, 512 1.25 -> 1.03, 1,021 3.48 -> 3.13; N S = 65,536
-// (four or two): 2,500 32.4 -> 30.9.
-int x_halves(int64_t N, int S) {
-    constexpr int64_t kSms = 152;
-    const int64_t one = ((N + kXP - 1) / kXP) * S, two = ((N + 2 * kXP - 1) / (2 * kXP)) * S;
-    const int64_t rounds1 = (one + kSms - 1) / kSms, rounds2 = (two + kSms - 1) / kSms;
-    return N > kXP && 10 * rounds1 >= 19 * rounds2 ? 2 : 1;
-}
-// Tiles of 128 points per shift, padded to whole CTAs: with N > 128 at most the
-// ceil(N / 64) sums a shift has room for.
-int64_t x_tiles(int64_t N, int S) {
-    const int64_t w = (int64_t)x_halves(N, S) * kXP;
-    return (N + w - 1) / w * (w / kXP);
-}
-
 template <int H>
 cudaError_t launch_x(const XArgs& a, int ctas, cudaStream_t st) {
     static std::mutex mu;
@@ -510,14 +486,20 @@ cudaError_t launch_x(const XArgs& a, int ctas, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+int current_sms() {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return device_sm_count(dev);
+}
+
 size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
 
 }  // namespace
 
 size_t full_fix_tc_scratch_bytes(int64_t D, int64_t N, int S) {
-    const int64_t nP = (D + kXB - 1) / kXB, nC = 2 * nP;
-    return al((size_t)nP * nC * kXChunkB) + al(sizeof(fix::Digits) * (size_t)nP * kXB * kXB) + al(sizeof(FixVar) * D) +
-           al((size_t)S * x_tiles(N, S) * nC * kXChunkA);
+    const FullFixPlan p = full_fix_plan(D, N, S, current_sms());
+    const int64_t nP = (D + kXB - 1) / kXB;
+    return al(p.tables) + al(sizeof(fix::Digits) * (size_t)nP * kXB * kXB) + al(sizeof(FixVar) * D) + al(p.history);
 }
 
 cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int64_t N, int S, const uint32_t* g,
@@ -527,7 +509,8 @@ cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int6
     const int64_t nP = (D + kXB - 1) / kXB, nC = 2 * nP;
     char* p = (char*)scratch;
     unsigned char* Lb = (unsigned char*)p;
-    p += al((size_t)nP * nC * kXChunkB);
+    const FullFixPlan plan = full_fix_plan(D, N, S, current_sms());
+    p += al(plan.tables);
     fix::Digits* Lp = (fix::Digits*)p;
     p += al(sizeof(fix::Digits) * (size_t)nP * kXB * kXB);
     FixVar* var = (FixVar*)p;
@@ -540,8 +523,7 @@ cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int6
     a.nP = (int)nP;
     a.nC = (int)nC;
     a.N = N;
-    const int halves = x_halves(N, S);
-    a.tps = (int)(x_tiles(N, S) / halves);
+    a.tps = (int)plan.per_shift;
     a.g = g;
     a.delta = delta;
     a.u = u;
@@ -556,7 +538,7 @@ cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int6
     a.wait_ns = (wait_ns > 0 && wait_ns < kXWaitNs) ? wait_ns : kXWaitNs;
     a.withhold = withhold;
     if (ev_begin && (e = cudaEventRecord(ev_begin, st)) != cudaSuccess) return e;
-    e = halves == 2 ? launch_x<2>(a, S * a.tps, st) : launch_x<1>(a, S * a.tps, st);
+    e = plan.halves == 2 ? launch_x<2>(a, (int)plan.ctas, st) : launch_x<1>(a, (int)plan.ctas, st);
     if (e == cudaSuccess && ev_end) e = cudaEventRecord(ev_end, st);
     return e;
 }
