@@ -319,10 +319,11 @@ int vecchia_mixture_log_cdf(vecchia_ctx* ctx, const double* sites_ordered, int64
  * the FP32 operands -- FP32-level accuracy --, FP64 running product and
  * sums).  log_p = log of the mean over shifts of the lattice means; rel_se =
  * their standard error over the mean.  Arrays host or device (both of one
- * kind); device memory grows as about 16 D^2 + 9.2 (mixed) or 16 (FP64: its
- * conditional means on the tensor cores too, exact sums of 64-bit fixed-point
- * products; 8 beyond 96 GB or where 16 does not fit, in integer products)
- * D S N bytes.  D <= VECCHIA_FULL_MAX_D.  A non-positive pivot gives
+ * kind); device memory grows as about 16 D^2 + 9.2 (mixed) or 8 (FP64) D S N
+ * bytes.  FP64 takes its conditional means on the tensor cores too from 64
+ * variables on (exact sums of 64-bit fixed-point products), in as many launches as
+ * keep to that, or to 24 D^2 bytes + 0.62 MB D where that is larger; where it does
+ * not fit, in integer products.  D <= VECCHIA_FULL_MAX_D.  A non-positive pivot gives
  * VECCHIA_ERR_NOT_PD with its site in vecchia_last_error_site();
  * VECCHIA_ERR_TIMEOUT means a bounded device wait of a tensor-core kernel ran
  * out (2 s without progress). */

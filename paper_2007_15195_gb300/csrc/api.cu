@@ -1391,9 +1391,9 @@ int vecchia_full_genz(vecchia_ctx* c, const double* sites, int64_t D, vecchia_co
     const size_t o_u = dv.off;
     if (!dev_in) dv.take<double>(D);
     const size_t o_scr = dv.off;
-    bool tc64 = !mixed && vk::full_fix_tc_pays(D, N, S);
+    bool tc64 = !mixed && vk::full_fix_tc_pays(D);
     int st = ensure_arena(c, o_scr + vk::full_genz_scratch_bytes(D, N, S, mixed, tc64));
-    if (st == VECCHIA_ERR_NOMEM && tc64) {  // the integer form keeps half the history
+    if (st == VECCHIA_ERR_NOMEM && tc64) {  // the integer form: no round of the other's fits
         tc64 = false;
         st = ensure_arena(c, o_scr + vk::full_genz_scratch_bytes(D, N, S, mixed, tc64));
     }

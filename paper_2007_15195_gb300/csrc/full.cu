@@ -30,13 +30,13 @@
 #include "cov.cuh"
 #include "exact_math.h"
 #include "fix_step.cuh"
+#include "full_fix_plan.h"
 #include "vk_internal.h"
 
 namespace vk {
 namespace {
 
 constexpr int kCholB = 32;   // Cholesky block
-constexpr int kFullP = 64;   // lattice points per CTA (FP64 recursion)
 constexpr int kFullKC = 32;  // history chunk of the contraction
 
 __global__ void full_cov_kernel(const double* __restrict__ sites, int D, CovParams cv, double* __restrict__ A) {
@@ -396,7 +396,7 @@ struct FullSmem {
 // triple against the FP64 fma's 76.  (Tiles of 128 points left 152 SMs with 1 or 2
 // tiles each at N S = 24,000.)  D = 1,021, N S = 24,000: 10.6 ms, D = 2,500, N S =
 // 65,536: 134 ms (490 in FP64); the tensor-core form takes 3.1 and 31 ms, so this one serves the
-// smallest problems and histories beyond kFixTcMaxBytes.
+// smallest problems and those for which the other's scratch cannot be had.
 __global__ void __launch_bounds__(kFullThreads) full_genz_kernel(const fix::Digits* __restrict__ Ld,
                                                                  const FixVar* __restrict__ var, FullArgs a,
                                                                  fix::Digits* __restrict__ Y,
@@ -778,14 +778,10 @@ int64_t full_genz_blocks_per_shift(int64_t N, bool mixed) {
 // status words) followed by the precision's own tables and y history.
 // FP64 recursion: the tensor cores' contraction from kFixTcMin variables on (N S =
 // 24,000: D = 64 0.08 against 0.16 ms, D = 256 0.39 against 0.94, D = 1,021 3.1
-// against 10.6), unless its history (16 bytes a y value, twice the integer form's)
-// would crowd out other work; the caller takes the integer form, too, where this
-// one's scratch cannot be allocated.
+// against 10.6); the caller takes the integer form, too, where this one's scratch
+// cannot be allocated.
 constexpr int64_t kFixTcMin = 64;
-constexpr size_t kFixTcMaxBytes = 96ull << 30;
-bool full_fix_tc_pays(int64_t D, int64_t N, int S) {
-    return D >= kFixTcMin && full_fix_tc_scratch_bytes(D, N, S) <= kFixTcMaxBytes;
-}
+bool full_fix_tc_pays(int64_t D) { return D >= kFixTcMin; }
 
 size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed, bool tc64) {
     const int64_t bps = (N + kFullP - 1) / kFullP, nblk = full_genz_blocks_per_shift(N, mixed);

@@ -82,6 +82,7 @@ struct XArgs {
     int D, nP, nC;              // variables, panels, chunks of 16
     int64_t N;
     int tps;                    // CTAs per shift
+    int64_t first;              // the launch's first CTA
     const uint32_t* g;          // lattice vector, D - 1 entries
     const double* delta;        // S x dim shifts
     const double* u;            // thresholds (for NaN only: its result is NaN)
@@ -89,7 +90,7 @@ struct XArgs {
     const FixVar* var;          // per variable (its bias counts the panel's own products)
     const unsigned char* Lb;    // digits of -L, [nP][nC] blocks of 8 KB (columns before the panel)
     const fix::Digits* Lp;      // [nP][32][32]: the panel's own triangle of -L
-    unsigned char* Y;           // history digits, [tiles][nC] chunks of 32 KB
+    unsigned char* Y;           // history digits, [the launch's tiles][nC] chunks of 32 KB
     double* part;               // per shift part_stride sums, the first H tps of them ours
     int part_stride;
     int* timeout;
@@ -313,7 +314,8 @@ __global__ void __launch_bounds__(kXThreads<H>, 1) full_fix_tc_kernel(XArgs a) {
     extern __shared__ __align__(1024) unsigned char x_smem[];
     XSmem<H>& sm = *reinterpret_cast<XSmem<H>*>(x_smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, D = a.D;
-    const int s = blockIdx.x / a.tps;
+    const int64_t cta = a.first + blockIdx.x;
+    const int s = (int)(cta / a.tps), tile = (int)(cta % a.tps);
     constexpr int kMmaWarp = H * kXP / 32, kCopyWarp = kMmaWarp + 1;
     unsigned char* Yt = a.Y + (int64_t)blockIdx.x * H * a.nC * kXChunkA;  // its halves' histories
     if (warp == kMmaWarp) {
@@ -332,7 +334,8 @@ __global__ void __launch_bounds__(kXThreads<H>, 1) full_fix_tc_kernel(XArgs a) {
             mbar_init(&sm.freed[i], kXP);
         }
         for (int h = 0; h < H; ++h) mbar_init(&sm.ydone[h], kXP);
-        sm.abort = sm.nan = 0;
+        sm.abort = *(const volatile int*)a.timeout;  // an earlier CTA gave up: so does this one
+        sm.nan = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     load_fix_tables(sm.tb);
@@ -346,7 +349,7 @@ __global__ void __launch_bounds__(kXThreads<H>, 1) full_fix_tc_kernel(XArgs a) {
         if (lane == 0) copy_all(a, sm, Yt);
     } else {
         const uint64_t K = fix::opaque_mid();
-        const int64_t k64 = (int64_t)(blockIdx.x % a.tps) * (H * kXP) + tid;
+        const int64_t k64 = (int64_t)tile * (H * kXP) + tid;
         const int h = tid / kXP, row = tid % kXP;
         const bool valid = k64 < a.N;
         const uint32_t k = (uint32_t)(valid ? k64 : a.N - 1);
@@ -457,7 +460,7 @@ __global__ void __launch_bounds__(kXThreads<H>, 1) full_fix_tc_kernel(XArgs a) {
         if (row == 0) {
             double t = 0.0;
             for (int w = 0; w < kXP / 32; ++w) t += sm.red[h * (kXP / 32) + w];
-            a.part[(int64_t)s * a.part_stride + (blockIdx.x % a.tps) * H + h] = sm.nan ? __longlong_as_double(0x7ff8000000000000LL) : t;
+            a.part[(int64_t)s * a.part_stride + (int64_t)tile * H + h] = sm.nan ? __longlong_as_double(0x7ff8000000000000LL) : t;
         }
     }
     tc_fence_before();
@@ -538,7 +541,10 @@ cudaError_t launch_full_fix_tc(const double* A, const double* u, int64_t D, int6
     a.wait_ns = (wait_ns > 0 && wait_ns < kXWaitNs) ? wait_ns : kXWaitNs;
     a.withhold = withhold;
     if (ev_begin && (e = cudaEventRecord(ev_begin, st)) != cudaSuccess) return e;
-    e = plan.halves == 2 ? launch_x<2>(a, (int)plan.ctas, st) : launch_x<1>(a, (int)plan.ctas, st);
+    for (a.first = 0; a.first < plan.ctas && e == cudaSuccess; a.first += plan.launch) {
+        const int n = (int)std::min(plan.launch, plan.ctas - a.first);
+        e = plan.halves == 2 ? launch_x<2>(a, n, st) : launch_x<1>(a, n, st);
+    }
     if (e == cudaSuccess && ev_end) e = cudaEventRecord(ev_end, st);
     return e;
 }

@@ -183,7 +183,7 @@ cudaError_t launch_conditioning(const double* L, int k, const double* sites_i, c
 // Cholesky, Genz over all variables; part_host gets S x ceil(N/128) tile sums
 // of the point products, *bad_host the first non-positive pivot (INT_MAX if none).
 // tc64: the FP64 recursion's contraction on the tensor cores (full_fix_tc_pays: worth it).
-bool full_fix_tc_pays(int64_t D, int64_t N, int S);
+bool full_fix_tc_pays(int64_t D);
 size_t full_genz_scratch_bytes(int64_t D, int64_t N, int S, bool mixed, bool tc64);
 // Point-block sums per shift written by launch_full_genz.
 int64_t full_genz_blocks_per_shift(int64_t N, bool mixed);
