@@ -390,6 +390,10 @@ int vecchia_set_tile(vecchia_ctx* ctx, int precision, int bucket, int warps, int
                      int slices, int groups);
 /* Back to the built-in tile rule for every precision and bucket. */
 int vecchia_reset_tiles(vecchia_ctx* ctx);
+/* The tile of that rule for a bucket of problems with `sites` terms in all, S
+ * shifts and N points: tile gets warps, points, slices, groups as vecchia_set_tile
+ * takes them (a launch of the tile equals the rule's). */
+int vecchia_builtin_tile(const vecchia_ctx* ctx, int precision, int bucket, int64_t sites, int S, int64_t N, int* tile);
 /* Record CUDA events around the Genz launches of each call (0 = off); for
  * vecchia_full_genz, around its recursion kernel alone. */
 int vecchia_set_timing(vecchia_ctx* ctx, int enable);

@@ -3,10 +3,11 @@
 A tile is (warps per CTA, points per lane, lattice slices per shift, shift
 groups per site): it changes only the launch shape, so results are identical
 for equal `slices` (and equal up to FP summation order otherwise).  The tuner
-times every candidate on the caller's own workload with the library's CUDA
-events around the Genz launches (vecchia_genz_time_ms), keeps the fastest,
-and caches it per (device, precision, bucket, N, S, size class) in a JSON file
-so later processes start from the tuned tile.
+times every candidate (by default the built-in rule's tile among them) on the
+caller's own workload with the library's CUDA events around the Genz launches
+(vecchia_genz_time_ms), keeps the fastest, and caches it per (device, precision,
+bucket, N, S, size class) in a JSON file so later processes start from the tuned
+tile.
 """
 import json
 import math
@@ -105,6 +106,11 @@ def tune(ctx, problems, precision=B.MIXED, candidates=None, reps=3, cache_path=N
     cands = list(candidates or DEFAULT_CANDIDATES)
     if precision == B.FP64:
         cands = sorted({(w, 1, s, g) for (w, p, s, g) in cands})
+    if not candidates:  # the rule that a tile takes the place of, for the largest block
+        bucket = max(bucket_of(int(p["m"]), int(p.get("group", 0))) for p in problems)
+        rule = B.vecchia_builtin_tile(ctx, precision, bucket, sum(int(p["sites"].shape[0]) for p in problems),
+                                      max(int(p["S"]) for p in problems), min(int(p["N"]) for p in problems))
+        cands = [rule] + [c for c in cands if c != rule]
     timings = []
     t0 = time.perf_counter()
     for tile in cands:

@@ -122,6 +122,7 @@ def lib():
         L.vecchia_last_error_site.argtypes = [_vp]
         L.vecchia_set_tile.argtypes = [_vp, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int]
         L.vecchia_reset_tiles.argtypes = [_vp]
+        L.vecchia_builtin_tile.argtypes = [_vp, C.c_int, C.c_int, C.c_int64, C.c_int, C.c_int64, C.POINTER(C.c_int)]
         L.vecchia_set_timing.argtypes = [_vp, C.c_int]
         L.vecchia_eval_special.argtypes = [_vp, C.c_int, _vp, C.c_int64, _vp]
         L.vecchia_eval_special64.argtypes = [_vp, C.c_int, _vp, C.c_int64, _vp]
@@ -541,6 +542,14 @@ def vecchia_set_tile(ctx, precision, bucket, warps, points, slices, groups):
 
 def vecchia_reset_tiles(ctx):
     _check(lib().vecchia_reset_tiles(ctx.handle), "vecchia_reset_tiles", ctx)
+
+
+def vecchia_builtin_tile(ctx, precision, bucket, sites, S, N):
+    """The built-in rule's (warps, points, slices, groups) for a bucket of problems."""
+    t = (C.c_int * 4)()
+    _check(lib().vecchia_builtin_tile(ctx.handle, int(precision), int(bucket), int(sites), int(S), int(N), t),
+           "vecchia_builtin_tile", ctx)
+    return tuple(t)
 
 
 def vecchia_eval_special(ctx, which, x):

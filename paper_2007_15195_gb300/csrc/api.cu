@@ -1971,6 +1971,19 @@ int vecchia_set_tile(vecchia_ctx* c, int precision, int bucket, int warps, int p
     return VECCHIA_OK;
 }
 
+int vecchia_builtin_tile(const vecchia_ctx* c, int precision, int bucket, int64_t sites, int S, int64_t N, int* tile) {
+    if (!c || !tile || (precision != VECCHIA_FP64 && precision != VECCHIA_MIXED) || bucket < 0 ||
+        bucket >= vk::kNumBuckets || sites < 1 || S < 2 || S > VECCHIA_MAX_S || N < 1)
+        return VECCHIA_ERR_ARG;
+    const bool mixed = precision == VECCHIA_MIXED;
+    const vk::GenzTile t = vk::default_tile(mixed, sites, S, bucket, vk::device_sm_count(c->device));
+    tile[0] = t.warps;
+    tile[1] = t.points;
+    tile[2] = vk::default_slices(mixed, S, N);
+    tile[3] = t.groups;
+    return VECCHIA_OK;
+}
+
 int vecchia_reset_tiles(vecchia_ctx* c) {
     if (!c) return VECCHIA_ERR_ARG;
     for (int p = 0; p < 2; ++p)

@@ -1259,6 +1259,8 @@ GenzTile default_tile(bool mixed, int64_t total_sites, int max_S, int bucket, in
     return t;
 }
 
+int default_slices(bool mixed, int S, int64_t N) { return auto_slices(S, N, mixed ? kModeFast : kModeFP64); }
+
 cudaError_t launch_genz(int bucket, bool mixed, const GenzTile& tile, const ProbDev* probs,
                         const int* seg_prefix, const int2* seg_base, int n_segs, int n_sites,
                         ProbResult* results, int* fallback_count, int2* fallback_items, int max_S,

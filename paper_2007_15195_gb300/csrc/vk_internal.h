@@ -87,6 +87,8 @@ struct GenzTile {
 
 // The built-in launch shape for a bucket of a batch (genz.cu).
 GenzTile default_tile(bool mixed, int64_t total_sites, int max_S, int bucket, int sms);
+// The lattice slices a shift that its slices = 0 stand for.
+int default_slices(bool mixed, int S, int64_t N);
 
 // ---------------- kernels' host launchers (genz.cu, knn.cu) ----------------
 
