@@ -99,8 +99,9 @@ int vecchia_set_stream(vecchia_ctx* ctx, void* cuda_stream);
  * host (MAXMIN: O(D^2) integer work over the host's cores).  With a context,
  * MAXMIN runs on the device (rounds of picks that no open site in reach
  * dominates, then a sort of their keys), with the same result; XY with both
- * arrays on the device runs there (a merge sort; on the host where its scratch
- * does not fit); the other cases run on the host.  MAXMIN: first the site nearest the centre of the quantised
+ * arrays on the device runs there (ranks by counting up to 8,192 sites, a merge
+ * sort beyond; on the host where its scratch does not fit); the other cases run
+ * on the host.  MAXMIN: first the site nearest the centre of the quantised
  * bounding box, then repeatedly the site farthest from the chosen ones, on
  * quantised coordinates, ties to the smaller index. */
 int vecchia_order(vecchia_ctx* ctx, const double* sites, int64_t D, int kind, int32_t* perm);
@@ -425,8 +426,10 @@ int vecchia_set_full_genz_wait(vecchia_ctx* ctx, uint64_t limit_ns, int withhold
  * (Sec. 2.2) in the precision the mixed path evaluates them. */
 int vecchia_eval_special(vecchia_ctx* ctx, int which, const float* x, int64_t n, float* out);
 
-/* Diagnostic: the FP64 special functions of the FP64 path on n values (x and
- * out device arrays of double): which = 0: Phi(x); 1: 1 - Phi(x) (from the
+/* Diagnostic: the FP64 special functions on the FP64 pipe, which the FP64 path
+ * takes below z = -7 and for probabilities below 2^-32 (its step evaluates the
+ * rest in 64-bit fixed point), on n values (x and out device arrays of double):
+ * which = 0: Phi(x); 1: 1 - Phi(x) (from the
  * tail); 2: Phi^{-1}(x) given p = x, q = 1 - x; 3: Phi^{-1}(1 - x) given q = x
  * (the upper tail, to full precision).  The same maps (Sec. 2.2) in FP64. */
 int vecchia_eval_special64(vecchia_ctx* ctx, int which, const double* x, int64_t n, double* out);

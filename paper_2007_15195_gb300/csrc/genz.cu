@@ -582,8 +582,9 @@ __device__ __forceinline__ void listed_item_of(const ItemSrc& src, int whole, in
 constexpr int kModeFP64 = 0, kModeFast = 1, kModeSafe = 2;
 
 // Register cap per thread: the FP64 step at up to 13 variables runs best with
-// 20 warps an SM (m = 10: 8.0 against 8.4 ms at 128 registers); from 14 on more
-// warps than 16 lose to spills.  The fast mixed loop keeps DMAX - 1 partial sums per
+// 20 warps an SM (m = 10: 8.0 against 8.4 ms at 128 registers); from 14 on 16 warps at
+// 128, spills and all (12 warps at 168 without: m = 24 18.06 against 18.12 ms, m = 27 21.97
+// against 21.32, m = 30 26.9 against 24.5).  The fast mixed loop keeps DMAX - 1 partial sums per
 // point in registers; capping the rest raises the number of resident warps.
 // Blocks above 32 variables run one point per lane with up to 128 registers
 // (fast) or 255 (FP64 and log-space forms, whose partial sums are wider), and

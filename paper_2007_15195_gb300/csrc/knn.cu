@@ -772,7 +772,7 @@ cudaError_t launch_sort(KEYS keys, int64_t D, int32_t* perm, const SortRun (&r)[
     return cudaGetLastError();
 }
 
-// ---- exact maxmin ordering (one thread-block cluster) -------------------------
+// ---- exact maxmin ordering (one thread-block cluster, or grid-wide rounds) ------
 // Same rule as the host ordering: first the site nearest the centre of the
 // quantised bounding box (2q - qmax, smallest squared distance, ties to the
 // smaller index), then repeatedly the unchosen site whose squared distance to

@@ -1,6 +1,6 @@
-// special_f64.h -- FP64 normal CDF and quantile on the FP64 pipe: a term's first
-// tails and vecchia_eval_special64 (the FP64 recursions take the same functions in
-// 64-bit fixed point, special_fix.h).
+// special_f64.h -- FP64 normal CDF and quantile on the FP64 pipe: the tail at z <= -7,
+// the quantile below 2^-32 (the rest of the FP64 recursions' functions is in 64-bit
+// fixed point, special_fix.h) and vecchia_eval_special64.
 //
 // GB300 runs FP64 at 1/64 of its FP32 rate, so these forms spend FP64
 // operations only where the value needs double precision and do the rest
@@ -22,7 +22,7 @@
 //     ~1e-15 relative (cubic convergence).
 //
 // The tables live in shared memory (Tables64, filled once per CTA), or stay in
-// global memory where a CTA reads them once (GlobalTables64).
+// global memory where they are read rarely (GlobalTables64).
 #pragma once
 
 #include <stdint.h>

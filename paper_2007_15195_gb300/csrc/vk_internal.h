@@ -134,11 +134,12 @@ constexpr int64_t kSmallMax = 512;
 cudaError_t launch_order_small(const double* sites, const double* u, int64_t D, int32_t* perm, double* sites_out,
                                double* u_out, void* scratch, cudaStream_t st);
 cudaError_t launch_knn_small(int64_t D, int m, int32_t* nbr, void* scratch, cudaStream_t st);
-// Exact maxmin ordering on the device (one thread-block cluster); perm (D, device)
-// gets new position -> old index; scratch from maxmin_scratch_bytes(D).
+// Exact maxmin ordering on the device (one thread-block cluster, from 6,000 sites on
+// after rounds over the whole GPU); perm (D, device) gets new position -> old index;
+// scratch from maxmin_scratch_bytes(D).
 size_t maxmin_scratch_bytes(int64_t D);
 cudaError_t launch_maxmin(const double* sites, int64_t D, int32_t* perm, void* scratch, cudaStream_t st);
-// XY ordering (x, then y, then index) of D device sites.
+// XY ordering (x, then y, then index) of D device sites: ranks by counting, or a merge sort.
 size_t order_xy_scratch_bytes(int64_t D);
 cudaError_t launch_order_xy(const double* sites, int64_t D, int32_t* perm, void* scratch, cudaStream_t st);
 // Union of the members' sets (per_site: D x m from launch_knn with group p)
